@@ -114,6 +114,7 @@ struct swm_ctx {
   int64_t nb = 0, nup = 0;
   int64_t* row_ptr = nullptr;  // [nw + 1]
   int32_t* col = nullptr;      // [nb]
+  int32_t* brow = nullptr;     // [nb] row p of block (p, q)
   int64_t* bt = nullptr;       // [nb] index of the transposed block
   int64_t* diag_b = nullptr;   // [nw] index of block (p, p)
   int64_t* ublk = nullptr;     // [nup] blocks (p, q) with q > p

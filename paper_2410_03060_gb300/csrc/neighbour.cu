@@ -105,7 +105,7 @@ struct RowCounts {
 };
 
 // mode 0: count kept partners per wire (and the sizes in RowCounts); mode 1: write them (sorted)
-// into col, with the position of each row's diagonal block and every block's first column in the
+// into col (and p into brow), with the position of each row's diagonal block and every block's first column in the
 // full layout and in the layout without the diagonal block (-1 for the diagonal).  One warp per wire: lanes 0..8 look up the nine (z, y) rows of three cells around the
 // wire's cell at once (each a contiguous range of the renumbered wires), a warp scan lays the
 // ranges end to end, and the warp tests 32 candidates per pass, so a wire costs about three
@@ -114,8 +114,8 @@ struct RowCounts {
 __global__ void k_pairs(int64_t nw, const double* __restrict__ cx, const double* __restrict__ cy,
                         const double* __restrict__ cz, const int32_t* __restrict__ cid, const int64_t* __restrict__ cstart,
                         Grid g, double rc2, int dense, int mode, RowCounts rc, const int32_t* __restrict__ m,
-                        const int64_t* __restrict__ row_ptr, int32_t* __restrict__ col, int64_t* __restrict__ diag_b,
-                        int32_t* __restrict__ colpos_f, int32_t* __restrict__ colpos_o) {
+                        const int64_t* __restrict__ row_ptr, int32_t* __restrict__ col, int32_t* __restrict__ brow,
+                        int64_t* __restrict__ diag_b, int32_t* __restrict__ colpos_f, int32_t* __restrict__ colpos_o) {
   const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (p >= nw) return;
@@ -189,6 +189,7 @@ __global__ void k_pairs(int64_t nw, const double* __restrict__ cx, const double*
       if (keep) {
         const int64_t b = base + count + __popc(bal & ((1u << lane) - 1u));
         col[b] = (int32_t)q;
+        brow[b] = (int32_t)p;
         const int32_t pf = kf + incl - mq;
         colpos_f[b] = pf;
         const bool diag_before = mp_seen || (dmask & ((1u << lane) - 1u));
@@ -234,45 +235,43 @@ __device__ __forceinline__ int64_t find_in_row(const int32_t* __restrict__ col, 
   return b;
 }
 
-__global__ void k_transpose_and_upper(int64_t nw, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                      const int64_t* __restrict__ diag_b, const int64_t* __restrict__ ubase,
-                                      int64_t* __restrict__ bt, int64_t* __restrict__ ublk) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= nw) return;
-  const int64_t b0 = row_ptr[p], b1 = row_ptr[p + 1];
-  for (int64_t b = b0; b < b1; ++b) {
-    const int32_t q = col[b];
-    bt[b] = find_in_row(col, row_ptr[q], row_ptr[q + 1], (int32_t)p);
-  }
-  int64_t u = ubase[p];
-  for (int64_t b = diag_b[p] + 1; b < b1; ++b) ublk[u++] = b;
-}
-
-// Column maps of both layouts (with and without the diagonal blocks), one thread per block-row.
-// Column maps of both layouts, and for the Krylov kernels each scalar row's wire and its 16-byte
-// descriptor in the off-diagonal layout (first value, first column-map entry, length).
-__global__ void k_colmap(int64_t nw, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                         const int32_t* __restrict__ m, const int64_t* __restrict__ off, Layout a, Layout b2,
-                         int32_t* __restrict__ rowwire, RowInfo* __restrict__ rinfo) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= nw) return;
-  {
+// Everything indexed by the kept blocks, one thread per block (p, q): the transposed block's index,
+// the list of blocks above the diagonal, the block's entries of the column maps of both layouts
+// (with and without the diagonal blocks), and, on the diagonal blocks, their wire's scalar rows:
+// the wire and the 16-byte descriptor in the off-diagonal layout (first value, first column-map
+// entry, length).  Bound by latency (a binary search of the partner's row); a thread per block
+// rather than per wire, because rows can be long: with 1,000 wires at entire coupling two kernels of
+// four CTAs, a thread per wire, took 2.3 and 1.7 ms side by side (the whole call 8.88 -> 7.25 ms); on
+// a 400,000-wire cloud the call went from 22.53 to 22.29 ms, on a 10,000-wire one 0.511 -> 0.500 ms.
+__global__ void __launch_bounds__(256) k_block_maps(int64_t nb, const int64_t* __restrict__ row_ptr,
+                                                    const int32_t* __restrict__ col, const int32_t* __restrict__ brow,
+                                                    const int64_t* __restrict__ diag_b,
+                                                    const int64_t* __restrict__ ubase, const int32_t* __restrict__ m,
+                                                    const int64_t* __restrict__ off, Layout a, Layout b2,
+                                                    int64_t* __restrict__ bt, int64_t* __restrict__ ublk,
+                                                    int32_t* __restrict__ rowwire, RowInfo* __restrict__ rinfo) {
+  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (b >= nb) return;
+  const int32_t p = brow[b], q = col[b];
+  const int32_t mq = m[q], oq = (int32_t)off[q];
+  const int32_t ca = a.colpos[b], cb = b2.colpos[b];
+  int32_t* ma = a.colmap + a.cmbase[p] + ca;
+  for (int j = 0; j < mq; ++j) ma[j] = oq + j;
+  if (p == q) {
+    bt[b] = b;
     const int K = b2.K[p];
-    const int64_t o0 = off[p], o1 = off[p + 1];
-    for (int64_t n = o0; n < o1; ++n) {
-      rowwire[n] = (int32_t)p;
-      rinfo[n] = RowInfo{b2.rowbase[p] + (n - o0) * K, (int32_t)b2.cmbase[p], K};
+    const int64_t o0 = off[p], vb = b2.rowbase[p];
+    const int32_t cm0 = (int32_t)b2.cmbase[p];
+    for (int i = 0; i < mq; ++i) {
+      rowwire[o0 + i] = p;
+      rinfo[o0 + i] = RowInfo{vb + (int64_t)i * K, cm0, K};
     }
+    return;
   }
-  for (int64_t b = row_ptr[p]; b < row_ptr[p + 1]; ++b) {
-    const int32_t q = col[b];
-    const int32_t ca = a.colpos[b], cb = b2.colpos[b];
-    for (int j = 0; j < m[q]; ++j) {
-      const int32_t v = (int32_t)(off[q] + j);
-      if (ca >= 0) a.colmap[a.cmbase[p] + ca + j] = v;
-      if (cb >= 0) b2.colmap[b2.cmbase[p] + cb + j] = v;
-    }
-  }
+  int32_t* mb = b2.colmap + b2.cmbase[p] + cb;
+  for (int j = 0; j < mq; ++j) mb[j] = oq + j;
+  bt[b] = find_in_row(col, row_ptr[q], row_ptr[q + 1], p);
+  if (q > p) ublk[ubase[p] + (b - diag_b[p] - 1)] = b;
 }
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)std::max<int64_t>(1, ceil_div(n, t)); }
@@ -395,7 +394,7 @@ int build_pattern(swm_ctx* ctx) {
   ctx->prof_begin(SWM_K_PAIRS);
   k_pairs<<<nblk(nw * 32, 256), 256, 0, st>>>(nw, ctx->cx, ctx->cy, ctx->cz, cid_s, cstart, g, rc2,
                                               ctx->dense ? 1 : 0, 0, rcs, m, nullptr, nullptr, nullptr, nullptr,
-                                              nullptr);
+                                              nullptr, nullptr);
   ctx->prof_end(SWM_K_PAIRS);
   SWM_LAUNCHED();
   {
@@ -422,20 +421,21 @@ int build_pattern(swm_ctx* ctx) {
   }
   if (ctx->nb > INT32_MAX / 2) return ctx->fail(SWM_EINVAL, "too many kept blocks for 32-bit positions");
   SWM_TRY(dalloc(ctx, B, (void**)&ctx->col, sizeof(int32_t) * ctx->nb));
+  SWM_TRY(dalloc(ctx, B, (void**)&ctx->brow, sizeof(int32_t) * ctx->nb));
   SWM_TRY(dalloc(ctx, B, (void**)&cpf, sizeof(int32_t) * ctx->nb));
   SWM_TRY(dalloc(ctx, B, (void**)&cpo, sizeof(int32_t) * ctx->nb));
   ctx->full.colpos = cpf;
   ctx->offd.colpos = cpo;
   ctx->prof_begin(SWM_K_PAIRS);
   k_pairs<<<nblk(nw * 32, 256), 256, 0, st>>>(nw, ctx->cx, ctx->cy, ctx->cz, cid_s, cstart, g, rc2,
-                                              ctx->dense ? 1 : 0, 1, rcs, m, ctx->row_ptr, ctx->col, ctx->diag_b,
+                                              ctx->dense ? 1 : 0, 1, rcs, m, ctx->row_ptr, ctx->col, ctx->brow, ctx->diag_b,
                                               cpf, cpo);
   ctx->prof_end(SWM_K_PAIRS);
   SWM_LAUNCHED();
 
-  // --- the transpose map with the upper-triangle block list, and the column maps on the build's
-  // second stream when it exists (both need the diagonal blocks and column positions that the
-  // writing pass of k_pairs produced)
+  // --- the transpose map with the upper-triangle block list, the column maps and the row
+  // descriptors (from the diagonal blocks and column positions that the writing pass of k_pairs
+  // produced)
   // the S-NFC pattern is symmetric, so the blocks above the diagonal are half the off-diagonal ones
   ctx->nup = (ctx->nb - nw) / 2;
   SWM_TRY(dalloc(ctx, B, (void**)&ctx->bt, sizeof(int64_t) * ctx->nb));
@@ -445,22 +445,10 @@ int build_pattern(swm_ctx* ctx) {
   if (ctx->offd.ncm > INT32_MAX) return ctx->fail(SWM_EINVAL, "column map too large for 32-bit offsets");
   SWM_TRY(dalloc(ctx, B, (void**)&ctx->rowwire, sizeof(int32_t) * std::max<int64_t>(1, ctx->N)));
   SWM_TRY(dalloc(ctx, B, &ctx->rowinfo, sizeof(RowInfo) * std::max<int64_t>(1, ctx->N)));
-  cudaStream_t s2 = ctx->side ? ctx->side : st;
-  if (ctx->side) {
-    SWM_CK(cudaEventRecord(ctx->side_ev[0], st));
-    SWM_CK(cudaStreamWaitEvent(s2, ctx->side_ev[0], 0));
-  }
-  // column maps (positions from the writing pass, offsets, multiplicities) and the row descriptors
-  k_colmap<<<nblk(nw, 256), 256, 0, s2>>>(nw, ctx->row_ptr, ctx->col, m, ctx->off, ctx->full, ctx->offd,
-                                          ctx->rowwire, (RowInfo*)ctx->rowinfo);
+  k_block_maps<<<nblk(ctx->nb, 256), 256, 0, st>>>(ctx->nb, ctx->row_ptr, ctx->col, ctx->brow, ctx->diag_b, ubase, m,
+                                                   ctx->off, ctx->full, ctx->offd, ctx->bt, ctx->ublk, ctx->rowwire,
+                                                   (RowInfo*)ctx->rowinfo);
   SWM_LAUNCHED();
-  k_transpose_and_upper<<<nblk(nw, 256), 256, 0, st>>>(nw, ctx->row_ptr, ctx->col, ctx->diag_b, ubase, ctx->bt,
-                                                       ctx->ublk);
-  SWM_LAUNCHED();
-  if (ctx->side) {
-    SWM_CK(cudaEventRecord(ctx->side_ev[1], s2));
-    SWM_CK(cudaStreamWaitEvent(st, ctx->side_ev[1], 0));
-  }
   ctx->m = m;
   dfree_group(ctx, tmp);
   return SWM_OK;
