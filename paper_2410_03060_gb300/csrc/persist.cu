@@ -45,6 +45,8 @@ constexpr int kPersistMaxRowsPerThread = 4;
 constexpr unsigned long long kBarrierNs = 1000000000ull;  // 1 s
 constexpr unsigned kBarrierMaxPolls = 1u << 26;            // second bound on a wait (>= 1.3 s of sleeps)
 constexpr int kPLanesPerRow = 4;                         // lanes per row of the persistent product
+constexpr int64_t kPersistWideRow = 128;  // mean entries per row from which a warp takes a row of E
+                                          // in global memory (four entries or more per lane)
 
 struct PArgs {
   KPtr P;                  // st, jlast, resid, H, coef, R, restart, N, tol
@@ -62,6 +64,7 @@ struct PArgs {
   int G, rows, max_iter;
   unsigned arrivals;       // arrivals a grid barrier waits for (G; more only in the timeout test)
   int vsm, esm;            // V / E slices in shared memory
+  int wide;                // long rows of E read from global memory: a warp per row
   int64_t emax, cmax;      // largest E and column-map slice of a CTA (entries)
   int bnorm_given;         // P.bnorm holds |b| (else the first residual norm is |b|)
   int y_zero;              // Y starts at zero: each CTA clears its rows and the first residual is B
@@ -402,6 +405,62 @@ __device__ void p_product(int mode, const PArgs& a, const ESlice<TV, TE>& S, con
           if (col[u] >= 0 && on[b]) S.xg[b * S.cstride + q0 + u * kPT] = v[u][b];
     }
     __syncthreads();
+  }
+  if (!S.xg && a.wide) {
+    // Long rows streamed from global memory (entire coupling: 5,128 entries a row at 1,000 wires,
+    // 210 MB of E per product): a warp per row, eight coalesced loads of E in flight per lane.
+    // Bound by HBM.  Four lanes per row read 32-byte pieces of eight rows: 0.63 ms per product
+    // there (8 steps 5.67 ms), 0.1 ms with a warp per row on every SM (8 steps 0.98 ms).
+    const int lane = threadIdx.x & 31;
+    for (int t = threadIdx.x >> 5; t < cnt; t += kPWarps) {
+      const RowInfo ri = S.ri[t];
+      const TE* e = S.e + (ri.vb - S.ebase);
+      const int32_t* cm = S.cm + (ri.cmb - S.cbase);
+      cplx<TV> acc[RB];
+#pragma unroll
+      for (int b = 0; b < RB; ++b) acc[b] = mkc<TV>(0, 0);
+      constexpr int U = 8;
+      int c = lane;
+      for (; c + (U - 1) * 32 < ri.K; c += U * 32) {
+        cplx<TV> ev[U];
+        int32_t cc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          ev[u] = ELoad<TV, TE>::ld(e + c + 32 * u);
+          cc[u] = cm[c + 32 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int b = 0; b < RB; ++b)
+            if (on[b]) cfma(acc[b], ev[u], ldcg_c<TV>(src + (int64_t)b * N + cc[u]));
+      }
+      for (; c < ri.K; c += 32) {
+        const cplx<TV> ev = ELoad<TV, TE>::ld(e + c);
+        const int64_t col = cm[c];
+#pragma unroll
+        for (int b = 0; b < RB; ++b)
+          if (on[b]) cfma(acc[b], ev, ldcg_c<TV>(src + (int64_t)b * N + col));
+      }
+      const int64_t n = n0 + t;
+#pragma unroll
+      for (int b = 0; b < RB; ++b) {
+        if (!on[b]) continue;
+        acc[b].re = warp_sum(acc[b].re);
+        acc[b].im = warp_sum(acc[b].im);
+        if (lane != 0) continue;
+        if (mode == 0) {
+          ws[b * a.rows + t] = ys[b * a.rows + t] + acc[b];
+        } else {
+          const cplx<TV> r = B[(int64_t)b * N + n] - (src[(int64_t)b * N + n] + acc[b]);
+          ys[b * a.rows + t] = r;
+          W[(int64_t)b * N + n] = r;
+          nrm[b] = fma(r.re, r.re, fma(r.im, r.im, nrm[b]));
+        }
+      }
+    }
+    if (mode == 1) p_norm_partials<TV, RB>(nrm, R, a.G, (TV*)a.partn, red);
+    return;
   }
   // four lanes per row, each taking every fourth entry, so that the rows of a dense part of the
   // cloud spread over the CTA's threads; passes over the rows are warp-uniform (quad sums below)
@@ -886,7 +945,12 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   const int R = P.R, restart = P.restart;
   const int64_t N = P.N;
   const int ctas = ctx->persist_ctas > 0 ? std::min(ctx->persist_ctas, std::max(ctx->nsm, 1)) : std::max(ctx->nsm, 1);
-  const int prows = (int)(ceil_div(ceil_div(std::max<int64_t>(N, 1), ctas), 32) * 32);
+  // Rows per CTA.  A multiple of 32 where a CTA's rows are few and short (fewer CTAs, cheaper
+  // barriers and sums); with long rows streamed from global memory every SM has to take its share
+  // (5,133 rows: 151 CTAs of 34 rows instead of 81 of 64).
+  const bool wide = ctx->offd.nval >= kPersistWideRow * N;
+  const int64_t rgran = wide ? 2 : 32;
+  const int prows = (int)(ceil_div(ceil_div(std::max<int64_t>(N, 1), ctas), rgran) * rgran);
   if (!(ctx->persist && ctx->coop && Bf.sync && R <= kPersistMaxR && N > 0 && N < ctx->split_rows &&
         prows <= kPersistMaxRowsPerThread * kPT))
     return SWM_OK;
@@ -935,6 +999,7 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   pa.max_iter = max_iter;
   pa.vsm = vsm;
   pa.esm = esm;
+  pa.wide = wide && !esm ? 1 : 0;
   pa.emax = emax;
   pa.cmax = cmax;
   pa.bnorm_given = Bf.bnorm_given;
