@@ -730,7 +730,7 @@ static int rcs_common(swm_ctx* ctx, int n_obs, const double* obs, bool mono, dou
   if (ctx->prec == SWM_C64) {
     rc = far_field_f32_launch(ctx, mono ? R : n_obs, obs_dev, stride, mono, sig, scratch, sb);
   } else {
-    rc = far_field_launch(ctx->stream, &ctx->launches, false, true, ctx->Xv, ctx->nw, ctx->N, nullptr, nullptr, ctx->cx,
+    rc = far_field_launch(ctx->stream, &ctx->launches, (const c128*)ctx->Xv, ctx->nw, ctx->N, nullptr, nullptr, ctx->cx,
                           ctx->cy, ctx->cz, ctx->tx, ctx->ty, ctx->tz, ctx->L, ctx->ns, ctx->off, true, ctx->k, R,
                           mono ? R : n_obs, obs_dev, stride, mono, sig, scratch, sb, &err);
     if (rc < 0) ctx->fail(rc, err);
@@ -954,7 +954,7 @@ static int far_field_common(void* cuda_stream, int64_t nw, const double* centres
     g_stateless_err = who + "scratch allocation failed";
     return SWM_ENOMEM;
   }
-  int rc = far_field_launch(st, nullptr, false, true, currents, nw, N, centres, dirs, nullptr, nullptr, nullptr,
+  int rc = far_field_launch(st, nullptr, (const c128*)currents, nw, N, centres, dirs, nullptr, nullptr, nullptr,
                             nullptr, nullptr, nullptr, lengths, nseg, off, false, k, n_rhs, n_obs, obs, 2, false,
                             sigma_out, scratch, sb, &g_stateless_err, components);
   cudaFreeAsync(scratch, st);

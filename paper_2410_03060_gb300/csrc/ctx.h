@@ -288,12 +288,11 @@ int far_field_alloc(swm_ctx* ctx);
 int prepare_far_field(swm_ctx* ctx, cudaStream_t s);
 int far_field_f32_launch(swm_ctx* ctx, int n_obs, const double* obs, int obs_stride, bool mono, double* sigma,
                          void* scratch, size_t scratch_bytes);
-int far_field_launch(cudaStream_t st, int64_t* launches, bool cur_c64, bool f64, const void* cur, int64_t nw,
-                     int64_t N, const double* c3, const double* t3, const double* cx, const double* cy,
-                     const double* cz, const double* tx, const double* ty, const double* tz, const double* Ls,
-                     const int32_t* ns, const int64_t* off, bool soa, double k, int n_rhs, int n_obs,
-                     const double* obs, int obs_stride, bool mono, double* sigma, void* scratch, size_t scratch_bytes,
-                     std::string* err, bool components = false);
+int far_field_launch(cudaStream_t st, int64_t* launches, const c128* cur, int64_t nw, int64_t N, const double* c3,
+                     const double* t3, const double* cx, const double* cy, const double* cz, const double* tx,
+                     const double* ty, const double* tz, const double* Ls, const int32_t* ns, const int64_t* off,
+                     bool soa, double k, int n_rhs, int n_obs, const double* obs, int obs_stride, bool mono,
+                     double* sigma, void* scratch, size_t scratch_bytes, std::string* err, bool components = false);
 // incidence frames on the host: k_hat (propagation, = -arrival) then polarisation e, 6 doubles each
 void frames_host(const double* inc, int n, std::vector<double>& out);
 // true if every pointer is device or managed memory (api.cu)

@@ -111,7 +111,7 @@ int far_noalloc_impl(void* cuda_stream, int64_t nw, const double* centres, const
     return SWM_ECUDA;
   }
   // every partial the reduction reads is written by this call, so nothing needs clearing
-  rc = far_field_launch(st, nullptr, false, true, currents, nw, N, centres, dirs, nullptr, nullptr, nullptr, nullptr,
+  rc = far_field_launch(st, nullptr, (const c128*)currents, nw, N, centres, dirs, nullptr, nullptr, nullptr, nullptr,
                         nullptr, nullptr, lengths, nseg, off, false, k, n_rhs, n_obs, obs, 2, false, sigma_out,
                         scratch, kNoAllocScratchBytes, err);
   if (rc < 0) return rc;
