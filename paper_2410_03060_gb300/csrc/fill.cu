@@ -23,6 +23,7 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "rhs_entry.cuh"
+#include "sincos64.cuh"
 
 namespace swm {
 
@@ -89,82 +90,118 @@ __device__ __forceinline__ void static_prims(R t, R al, R out[4]) {
   out[3] = (t * t - R(2) * al * al) * r / R(3);
 }
 
-// I[ab] for segment offset d >= 0 of a wire with segment length D and radius a (without 1/(4 pi)),
-// in precision R.  xg, wg: 8-point Gauss-Legendre rule on [0, 1].
+// Per-CTA tables of the self blocks in precision R: the Gauss nodes, the weights times the shape
+// convolutions at the nodes, and the convolutions' coefficients, formed in R once per CTA.  (The
+// coefficients are float64 constants: converting them at each use issues about sixteen times slower
+// than a float32 instruction.)
 template <typename R>
-__device__ void self_offset(int d, R D, R a, R k, const R* xg, const R* wg, cplx<R> out[4]) {
+struct SelfTab {
+  R x[8], ww[2][8][4], poly[2][4][4];
+  __device__ void fill(const GLTable& gl) {
+    for (int e = threadIdx.x; e < 64; e += blockDim.x) {
+      const int half = e >> 5, g = (e >> 2) & 7, ab = e & 3;
+      const double* P = c_self_poly[half][ab];
+      const R w = (half ? R(0) : R(-1)) + (R)gl.x8[g], wg = (R)gl.w8[g];
+      ww[half][g][ab] = wg * (((R(P[3]) * w + R(P[2])) * w + R(P[1])) * w + R(P[0]));
+    }
+    for (int e = threadIdx.x; e < 32; e += blockDim.x) poly[e >> 4][(e >> 2) & 3][e & 3] = (R)c_self_poly[e >> 4][(e >> 2) & 3][e & 3];
+    for (int e = threadIdx.x; e < 8; e += blockDim.x) x[e] = (R)gl.x8[e];
+    __syncthreads();
+  }
+};
+
+// The share of halves h0 .. h1 - 1 of I[ab] for segment offset d >= 0 of a wire with segment length D
+// and radius a (without 1/(4 pi)), in precision R.
+template <typename R>
+__device__ __forceinline__ void self_offset(int d, int h0, int h1, R D, R a, R k, const SelfTab<R>& tab,
+                                            cplx<R> out[4]) {
   for (int ab = 0; ab < 4; ++ab) out[ab] = mkc<R>(0, 0);
   const R al = a / D;
-  for (int half = 0; half < 2; ++half) {
-    const R w0 = half ? R(0) : R(-1);
-    for (int g = 0; g < 8; ++g) {
-      const R w = w0 + xg[g];
-      const R t = R(d) + w;
-      const R Rr = sqrt(D * D * t * t + a * a);
-      // half-angle form keeps cos(kR) - 1 accurate when kR is small
-      R sh, ch;
+  for (int half = h0; half < h1; ++half) {
+  const R w0 = half ? R(0) : R(-1);
+  for (int g = 0; g < 8; ++g) {
+    const R w = w0 + tab.x[g];
+    const R t = R(d) + w;
+    const R R2 = D * D * t * t + a * a;
+    // half-angle form keeps cos(kR) - 1 accurate when kR is small; the full kernel exp(-jkR)/R, or the
+    // smooth remainder (exp(-jkR) - 1)/R for |d| <= 1
+    R sh, ch, re, im;
+    if constexpr (sizeof(R) == 8) {
+      const R ri = rsqrt(R2);
+      sincos_table(0.5 * k * (R2 * ri), &sh, &ch);
+      const R s2 = sh + sh, cm1 = -s2 * sh;
+      re = (d <= 1 ? cm1 : R(1) + cm1) * ri;
+      im = -s2 * ch * ri;
+    } else {
+      const R Rr = sqrt(R2);
       sincos(R(0.5) * k * Rr, &sh, &ch);
       const R cm1 = R(-2) * sh * sh, sn = R(2) * sh * ch;
-      // full kernel exp(-jkR)/R, or the smooth remainder (exp(-jkR) - 1)/R for |d| <= 1
-      const R re = (d <= 1 ? cm1 : R(1) + cm1) / Rr, im = -sn / Rr;
-      const R ww = wg[g];
-      for (int ab = 0; ab < 4; ++ab) {
-        const double* P = c_self_poly[half][ab];
-        const R W = ((R(P[3]) * w + R(P[2])) * w + R(P[1])) * w + R(P[0]);
-        out[ab].re += ww * W * re;
-        out[ab].im += ww * W * im;
-      }
+      re = (d <= 1 ? cm1 : R(1) + cm1) / Rr;
+      im = -sn / Rr;
     }
-    if (d <= 1) {
-      // static part: int W(t - d) / (D sqrt(t^2 + al^2)) dt over t in [w0 + d, w0 + 1 + d]
-      R A0[4], A1[4];
-      static_prims<R>(w0 + R(d), al, A0);
-      static_prims<R>(w0 + R(1) + R(d), al, A1);
-      for (int ab = 0; ab < 4; ++ab) {
-        const double* P = c_self_poly[half][ab];
-        // coefficients of W(t - d) in powers of t
-        const R dd = (R)d;
-        const R q0 = R(P[0]) - R(P[1]) * dd + R(P[2]) * dd * dd - R(P[3]) * dd * dd * dd;
-        const R q1 = R(P[1]) - R(2) * R(P[2]) * dd + R(3) * R(P[3]) * dd * dd;
-        const R q2 = R(P[2]) - R(3) * R(P[3]) * dd;
-        const R q3 = R(P[3]);
-        const R st = q0 * (A1[0] - A0[0]) + q1 * (A1[1] - A0[1]) + q2 * (A1[2] - A0[2]) + q3 * (A1[3] - A0[3]);
-        out[ab].re += st / D;
-      }
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+      const R W = tab.ww[half][g][ab];
+      out[ab].re += W * re;
+      out[ab].im += W * im;
     }
+  }
+  if (d <= 1) {
+    // static part: int W(t - d) / (D sqrt(t^2 + al^2)) dt over t in [w0 + d, w0 + 1 + d]
+    R A0[4], A1[4];
+    static_prims<R>(w0 + R(d), al, A0);
+    static_prims<R>(w0 + R(1) + R(d), al, A1);
+    for (int ab = 0; ab < 4; ++ab) {
+      const R* P = tab.poly[half][ab];
+      // coefficients of W(t - d) in powers of t
+      const R dd = (R)d;
+      const R q0 = P[0] - P[1] * dd + P[2] * dd * dd - P[3] * dd * dd * dd;
+      const R q1 = P[1] - R(2) * P[2] * dd + R(3) * P[3] * dd * dd;
+      const R q2 = P[2] - R(3) * P[3] * dd;
+      const R q3 = P[3];
+      const R st = q0 * (A1[0] - A0[0]) + q1 * (A1[1] - A0[1]) + q2 * (A1[2] - A0[2]) + q3 * (A1[3] - A0[3]);
+      out[ab].re += st / D;
+    }
+  }
   }
   for (int ab = 0; ab < 4; ++ab) out[ab] = (D * D) * out[ab];
 }
 
-constexpr int kSelfThreads = 128;
+constexpr int kSelfThreads = 64;
 
-// One thread per (wire, segment offset d >= 0): S slots per wire (S a power of two >= max n_s),
-// kSelfThreads / S wires per CTA; then the CTA writes the Toeplitz blocks of its wires.
+// One thread per (wire, segment offset d >= 0), in float64 one per half of it with the halves added by a
+// shuffle (float64 issue sets the time, so a small cloud's work is spread over more warps): S slots of
+// SPLIT threads per wire (S a power of two >= max n_s); then the CTA writes the Toeplitz blocks of its
+// wires.
 template <typename R, typename TV>
 __global__ void __launch_bounds__(kSelfThreads) k_self_blocks(int64_t nw, const double* __restrict__ Ls,
                                                              const double* __restrict__ as,
                                                              const int32_t* __restrict__ ns, double k, GLTable gl,
                                                              const int64_t* __restrict__ diag_b, Layout lay, int S,
                                                              cplx<TV>* __restrict__ Z) {
-  __shared__ cplx<R> sI[kSelfThreads][4];
-  __shared__ int obase[kSelfThreads + 1];
-  __shared__ R xg[8], wg[8];
-  const int wpc = kSelfThreads / S;
+  constexpr int SPLIT = sizeof(R) == 8 ? 2 : 1;
+  __shared__ cplx<R> sI[kSelfThreads / SPLIT][4];
+  __shared__ int obase[kSelfThreads / SPLIT + 1];
+  __shared__ SelfTab<R> tab;
+  const int wpc = kSelfThreads / (SPLIT * S);
   const int64_t p0 = (int64_t)blockIdx.x * wpc;
   const int tid = threadIdx.x;
-  if (tid < 8) {
-    xg[tid] = (R)gl.x8[tid];
-    wg[tid] = (R)gl.w8[tid];
-  }
-  __syncthreads();
+  tab.fill(gl);
   {
-    const int lw = tid / S, d = tid % S;
+    const int lw = tid / (SPLIT * S), d = (tid / SPLIT) % S, half = tid % SPLIT;
     const int64_t p = p0 + lw;
-    if (p < nw && d < ns[p]) {
-      cplx<R> I[4];
-      self_offset<R>(d, (R)(Ls[p] / ns[p]), (R)as[p], (R)k, xg, wg, I);
-      for (int ab = 0; ab < 4; ++ab) sI[tid][ab] = I[ab];
+    const bool on = lw < wpc && p < nw && d < ns[p];
+    cplx<R> I[4] = {};
+    if (on) self_offset<R>(d, half, SPLIT == 2 ? half + 1 : 2, (R)(Ls[p] / ns[p]), (R)as[p], (R)k, tab, I);
+    if constexpr (SPLIT == 2) {
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        I[ab].re += __shfl_xor_sync(0xffffffffu, I[ab].re, 1);
+        I[ab].im += __shfl_xor_sync(0xffffffffu, I[ab].im, 1);
+      }
     }
+    if (on && half == 0)
+      for (int ab = 0; ab < 4; ++ab) sI[tid / SPLIT][ab] = I[ab];
   }
   if (tid == 0) {
     int acc = 0;
@@ -206,13 +243,11 @@ __global__ void __launch_bounds__(kSelfThreads) k_self_blocks(int64_t nw, const 
 // mutual blocks
 
 struct BlockGeo {
-  float D[3], tp[3], tq[3];  // FP32 copies (fast path); the FP64 path re-reads FP64 geometry
-  float Lp, Lq, a2, tpq;
-  float f, sc;               // D_p D_q / (4 pi) and 1 / (k^2 D_p D_q), formed in float64
-  double fd, scd, tpqd;      // the same in float64 for the float64 path
+  double D[3], tp[3], tq[3];
+  double Lp, Lq, Dp, Dq, a2, tpq;
+  double f, sc;              // D_p D_q / (4 pi) and 1 / (k^2 D_p D_q)
   int nsp, nsq, nq, item0;   // item0: first segment pair of this block in the batch
   int out0;                  // first output entry of this block in the batch
-  int p, q;
   int64_t bpq, bqp;          // value offsets of Z_pq[0][0] and Z_qp[0][0]
   int Kp, Kq;
 };
@@ -251,98 +286,51 @@ struct SegI {
   cplx<R> rr, rf, fr, ff;
 };
 
-// Shape integrals of one segment pair (without the 1/(4 pi) D_p D_q factor).
+// Shape integrals of one segment pair (without the 1/(4 pi) D_p D_q factor), float64.  xg, wg the nodes and weights, wx = wg xg.  Bound by float64 issue, so instructions are
+// what counts: 1/R from rsqrt, sine and cosine from the table, the points of wire q once per segment
+// pair: about 35 float64 instructions per kernel value against about 90 with sqrt, two divisions and
+// CUDA's sincos.
 template <int NQ>
-__device__ __forceinline__ void seg_pair_f32(const BlockGeo& G, int u, int v, float k, const float* xg, const float* wg,
-                                             SegI<float>& out) {
-  float Ex[NQ], Ey[NQ], Ez[NQ], Qx[NQ], Qy[NQ], Qz[NQ];
-  const float Dp = G.Lp / G.nsp, Dq = G.Lq / G.nsq;
+__device__ __forceinline__ void seg_pair_f64(const BlockGeo& G, int u, int v, double k, const double* xg,
+                                             const double* wg, const double* wx, SegI<double>& out) {
+  double Qx[NQ], Qy[NQ], Qz[NQ];
 #pragma unroll
-  for (int g = 0; g < NQ; ++g) {
-    const float sp = -0.5f * G.Lp + ((float)u + xg[g]) * Dp;
-    Ex[g] = G.D[0] + sp * G.tp[0];
-    Ey[g] = G.D[1] + sp * G.tp[1];
-    Ez[g] = G.D[2] + sp * G.tp[2];
-    const float sq = -0.5f * G.Lq + ((float)v + xg[g]) * Dq;
-    Qx[g] = sq * G.tq[0];
-    Qy[g] = sq * G.tq[1];
-    Qz[g] = sq * G.tq[2];
+  for (int h = 0; h < NQ; ++h) {
+    const double sq = -0.5 * G.Lq + (v + xg[h]) * G.Dq;
+    Qx[h] = sq * G.tq[0];
+    Qy[h] = sq * G.tq[1];
+    Qz[h] = sq * G.tq[2];
   }
-  float rrr = 0.f, rri = 0.f, rfr = 0.f, rfi = 0.f, frr = 0.f, fri = 0.f, ffr = 0.f, ffi = 0.f;
-#pragma unroll
-  for (int g = 0; g < NQ; ++g) {
-    float Ar = 0.f, Ai = 0.f, Br = 0.f, Bi = 0.f;
-#pragma unroll
-    for (int h = 0; h < NQ; ++h) {
-      const float dx = Ex[g] - Qx[h], dy = Ey[g] - Qy[h], dz = Ez[g] - Qz[h];
-      const float R2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, G.a2)));
-      const float ri = rsqrtf(R2);
-      const float Rr = R2 * ri;
-      float s, c;
-      __sincosf(k * Rr, &s, &c);
-      const float gr = c * ri, gi = -s * ri;
-      const float wh = wg[h], wxh = wg[h] * xg[h];
-      Ar = fmaf(wh, gr, Ar);
-      Ai = fmaf(wh, gi, Ai);
-      Br = fmaf(wxh, gr, Br);
-      Bi = fmaf(wxh, gi, Bi);
-    }
-    const float wr = wg[g] * xg[g], wf = wg[g] - wr;
-    const float Cr = Ar - Br, Ci = Ai - Bi;
-    rrr = fmaf(wr, Br, rrr);
-    rri = fmaf(wr, Bi, rri);
-    rfr = fmaf(wr, Cr, rfr);
-    rfi = fmaf(wr, Ci, rfi);
-    frr = fmaf(wf, Br, frr);
-    fri = fmaf(wf, Bi, fri);
-    ffr = fmaf(wf, Cr, ffr);
-    ffi = fmaf(wf, Ci, ffi);
-  }
-  out.rr = mkc(rrr, rri);
-  out.rf = mkc(rfr, rfi);
-  out.fr = mkc(frr, fri);
-  out.ff = mkc(ffr, ffi);
-}
-
-template <int NQ>
-__device__ __forceinline__ void seg_pair_f64(const double* __restrict__ cx, const double* __restrict__ cy,
-                                             const double* __restrict__ cz, const double* __restrict__ tx,
-                                             const double* __restrict__ ty, const double* __restrict__ tz,
-                                             const double* __restrict__ Ls, const double* __restrict__ as,
-                                             const BlockGeo& G, int u, int v, double k, const double* xg,
-                                             const double* wg, SegI<double>& out) {
-  const int p = G.p, q = G.q;
-  const double D[3] = {cx[p] - cx[q], cy[p] - cy[q], cz[p] - cz[q]};
-  const double tp[3] = {tx[p], ty[p], tz[p]}, tq[3] = {tx[q], ty[q], tz[q]};
-  const double Lp = Ls[p], Lq = Ls[q];
-  const double a2 = 0.5 * (as[p] * as[p] + as[q] * as[q]);
-  const double Dp = Lp / G.nsp, Dq = Lq / G.nsq;
   double rrr = 0, rri = 0, rfr = 0, rfi = 0, frr = 0, fri = 0, ffr = 0, ffi = 0;
+#pragma unroll 1
   for (int g = 0; g < NQ; ++g) {
-    const double sp = -0.5 * Lp + (u + xg[g]) * Dp;
-    const double Ex = D[0] + sp * tp[0], Ey = D[1] + sp * tp[1], Ez = D[2] + sp * tp[2];
-    double Ar = 0, Ai = 0, Br = 0, Bi = 0;
+    const double sp = -0.5 * G.Lp + (u + xg[g]) * G.Dp;
+    const double Ex = G.D[0] + sp * G.tp[0], Ey = G.D[1] + sp * G.tp[1], Ez = G.D[2] + sp * G.tp[2];
+    double Ar = 0, As = 0, Br = 0, Bs = 0;
+#pragma unroll
     for (int h = 0; h < NQ; ++h) {
-      const double sq = -0.5 * Lq + (v + xg[h]) * Dq;
-      const double dx = Ex - sq * tq[0], dy = Ey - sq * tq[1], dz = Ez - sq * tq[2];
-      const double R = sqrt(dx * dx + dy * dy + dz * dz + a2);
+      const double dx = Ex - Qx[h], dy = Ey - Qy[h], dz = Ez - Qz[h];
+      const double R2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, G.a2)));
+      const double ri = rsqrt(R2);
       double s, c;
-      sincos(k * R, &s, &c);
-      const double gr = c / R, gi = -s / R;
-      Ar += wg[h] * gr;
-      Ai += wg[h] * gi;
-      Br += wg[h] * xg[h] * gr;
-      Bi += wg[h] * xg[h] * gi;
+      sincos_table(k * (R2 * ri), &s, &c);
+      const double gr = c * ri, gs = s * ri;
+      Ar = fma(wg[h], gr, Ar);
+      As = fma(wg[h], gs, As);
+      Br = fma(wx[h], gr, Br);
+      Bs = fma(wx[h], gs, Bs);
     }
-    const double wr = wg[g] * xg[g], wf = wg[g] - wr;
-    rrr += wr * Br;
-    rri += wr * Bi;
-    rfr += wr * (Ar - Br);
-    rfi += wr * (Ai - Bi);
-    frr += wf * Br;
-    fri += wf * Bi;
-    ffr += wf * (Ar - Br);
-    ffi += wf * (Ai - Bi);
+    // G = (cos - j sin) / R: the imaginary parts are minus the sine sums
+    const double wr = wx[g], wf = wg[g] - wr;
+    const double Cr = Ar - Br, Cs = As - Bs;
+    rrr = fma(wr, Br, rrr);
+    rri = fma(-wr, Bs, rri);
+    rfr = fma(wr, Cr, rfr);
+    rfi = fma(-wr, Cs, rfi);
+    frr = fma(wf, Br, frr);
+    fri = fma(-wf, Bs, fri);
+    ffr = fma(wf, Cr, ffr);
+    ffi = fma(-wf, Cs, ffi);
   }
   out.rr = mkc(rrr, rri);
   out.rf = mkc(rfr, rfi);
@@ -350,19 +338,21 @@ __device__ __forceinline__ void seg_pair_f64(const double* __restrict__ cx, cons
   out.ff = mkc(ffr, ffi);
 }
 
-constexpr int kFillThreads = 256;
+constexpr int kFillThreads = 128;
 
 __host__ __device__ constexpr size_t round16(size_t x) { return (x + 15) / 16 * 16; }
 
-// One CTA per batch of `nbatch` upper blocks.  Shared memory: BlockGeo[nbatch], item and output
-// prefix arrays, and SegI<R> for every segment pair of the batch (capacity `cap`).
-template <typename R, typename TV>
-__global__ void __launch_bounds__(kFillThreads, sizeof(R) == 4 ? 3 : 1) k_mutual_blocks(
-    int64_t nup, const int64_t* __restrict__ ublk, const int32_t* __restrict__ col, const int64_t* __restrict__ bt,
-    const double* __restrict__ cx, const double* __restrict__ cy, const double* __restrict__ cz,
-    const double* __restrict__ tx, const double* __restrict__ ty, const double* __restrict__ tz,
-    const double* __restrict__ Ls, const double* __restrict__ as, const int32_t* __restrict__ ns, double k,
-    GLTable gl, Layout lay, int nbatch, cplx<TV>* __restrict__ Z, unsigned long long* __restrict__ evals) {
+// One CTA per batch of `nbatch` upper blocks (float64 path).  Shared memory: BlockGeo[nbatch], item and
+// output prefix arrays, and the shape integrals of every segment pair of the batch.  The host takes
+// batches small enough to give every SM a few CTAs (221 blocks of a 200-wire cloud in batches of one
+// instead of 16 in 14 CTAs: 328 -> 34 us; 69,205 blocks of a clustered cloud 2.51 -> 1.55 ms).
+__global__ void __launch_bounds__(kFillThreads) k_mutual_blocks_f64(
+    int64_t nup, const int64_t* __restrict__ ublk, const int32_t* __restrict__ col, const int32_t* __restrict__ brow,
+    const int64_t* __restrict__ bt, const double* __restrict__ cx, const double* __restrict__ cy,
+    const double* __restrict__ cz, const double* __restrict__ tx, const double* __restrict__ ty,
+    const double* __restrict__ tz, const double* __restrict__ Ls, const double* __restrict__ as,
+    const int32_t* __restrict__ ns, double k, GLTable gl, Layout lay, int nbatch, c128* __restrict__ Z,
+    unsigned long long* __restrict__ evals) {
   extern __shared__ __align__(16) unsigned char smem[];
   const size_t o_item = round16(sizeof(BlockGeo) * nbatch);
   const size_t o_out = o_item + round16(sizeof(int) * (nbatch + 1));
@@ -370,35 +360,37 @@ __global__ void __launch_bounds__(kFillThreads, sizeof(R) == 4 ? 3 : 1) k_mutual
   BlockGeo* geo = reinterpret_cast<BlockGeo*>(smem);
   int* item_pre = reinterpret_cast<int*>(smem + o_item);  // nbatch + 1
   int* out_pre = reinterpret_cast<int*>(smem + o_out);    // nbatch + 1
-  SegI<R>* seg = reinterpret_cast<SegI<R>*>(smem + o_seg);
-  __shared__ float xs4[4], ws4[4], xs8[8], ws8[8];
+  SegI<double>* seg = reinterpret_cast<SegI<double>*>(smem + o_seg);
+  __shared__ double x4[4], w4[4], wx4[4], x8[8], w8[8], wx8[8];
   __shared__ unsigned long long cta_evals;
 
   const int tid = threadIdx.x;
   const int64_t b0 = (int64_t)blockIdx.x * nbatch;
   const int nb_here = (int)min((int64_t)nbatch, nup - b0);
   if (tid < 4) {
-    xs4[tid] = (float)gl.x4[tid];
-    ws4[tid] = (float)gl.w4[tid];
+    x4[tid] = gl.x4[tid];
+    w4[tid] = gl.w4[tid];
+    wx4[tid] = gl.w4[tid] * gl.x4[tid];
   }
   if (tid < 8) {
-    xs8[tid] = (float)gl.x8[tid];
-    ws8[tid] = (float)gl.w8[tid];
+    x8[tid] = gl.x8[tid];
+    w8[tid] = gl.w8[tid];
+    wx8[tid] = gl.w8[tid] * gl.x8[tid];
   }
   if (tid == 0) cta_evals = 0;
   __syncthreads();
-  // --- per-block setup, float64, one thread per block
+  // --- per-block setup, one thread per block
   if (tid < nb_here) {
     const int64_t b = ublk[b0 + tid];
-    const int q = col[b];
+    const int q = col[b], p = brow[b];
     const int64_t bq = bt[b];
-    const int p = col[bq];
     BlockGeo G;
     const double D[3] = {cx[p] - cx[q], cy[p] - cy[q], cz[p] - cz[q]};
     const double tp[3] = {tx[p], ty[p], tz[p]}, tq[3] = {tx[q], ty[q], tz[q]};
     const double Lp = Ls[p], Lq = Ls[q];
     const int nsp = ns[p], nsq = ns[q];
-    const double dmax = fmax(Lp / nsp, Lq / nsq);
+    const double Dp = Lp / nsp, Dq = Lq / nsq;
+    const double dmax = fmax(Dp, Dq);
     // near rule: exact segment distance < longer segment length; skipped when the centroid
     // distance already exceeds half the two lengths plus that length
     int nq = 4;
@@ -408,27 +400,21 @@ __global__ void __launch_bounds__(kFillThreads, sizeof(R) == 4 ? 3 : 1) k_mutual
       if (seg_dist(D, tp, 0.5 * Lp, tq, 0.5 * Lq) < dmax) nq = 8;
     }
     for (int c = 0; c < 3; ++c) {
-      G.D[c] = (float)D[c];
-      G.tp[c] = (float)tp[c];
-      G.tq[c] = (float)tq[c];
+      G.D[c] = D[c];
+      G.tp[c] = tp[c];
+      G.tq[c] = tq[c];
     }
-    G.Lp = (float)Lp;
-    G.Lq = (float)Lq;
-    G.a2 = (float)(0.5 * (as[p] * as[p] + as[q] * as[q]));
-    G.tpqd = tp[0] * tq[0] + tp[1] * tq[1] + tp[2] * tq[2];
-    G.tpq = (float)G.tpqd;
-    {
-      const double Dp = Lp / nsp, Dq = Lq / nsq;
-      G.fd = Dp * Dq / kFourPi;
-      G.scd = 1.0 / (k * k * Dp * Dq);
-      G.f = (float)G.fd;
-      G.sc = (float)G.scd;
-    }
+    G.Lp = Lp;
+    G.Lq = Lq;
+    G.Dp = Dp;
+    G.Dq = Dq;
+    G.a2 = 0.5 * (as[p] * as[p] + as[q] * as[q]);
+    G.tpq = tp[0] * tq[0] + tp[1] * tq[1] + tp[2] * tq[2];
+    G.f = Dp * Dq / kFourPi;
+    G.sc = 1.0 / (k * k * Dp * Dq);
     G.nsp = nsp;
     G.nsq = nsq;
     G.nq = nq;
-    G.p = p;
-    G.q = q;
     G.Kp = lay.K[p];
     G.Kq = lay.K[q];
     G.bpq = lay.rowbase[p] + lay.colpos[b];
@@ -467,18 +453,11 @@ __global__ void __launch_bounds__(kFillThreads, sizeof(R) == 4 ? 3 : 1) k_mutual
     const BlockGeo& G = geo[lo];
     const int local = it - G.item0;
     const int u = local / G.nsq, v = local % G.nsq;
-    SegI<R> s;
-    if constexpr (sizeof(R) == 4) {
-      if (G.nq == 4)
-        seg_pair_f32<4>(G, u, v, (float)k, xs4, ws4, s);
-      else
-        seg_pair_f32<8>(G, u, v, (float)k, xs8, ws8, s);
-    } else {
-      if (G.nq == 4)
-        seg_pair_f64<4>(cx, cy, cz, tx, ty, tz, Ls, as, G, u, v, k, gl.x4, gl.w4, s);
-      else
-        seg_pair_f64<8>(cx, cy, cz, tx, ty, tz, Ls, as, G, u, v, k, gl.x8, gl.w8, s);
-    }
+    SegI<double> s;
+    if (G.nq == 4)
+      seg_pair_f64<4>(G, u, v, k, x4, w4, wx4, s);
+    else
+      seg_pair_f64<8>(G, u, v, k, x8, w8, wx8, s);
     seg[it] = s;
   }
   __syncthreads();
@@ -498,28 +477,17 @@ __global__ void __launch_bounds__(kFillThreads, sizeof(R) == 4 ? 3 : 1) k_mutual
     const int mq = G.nsq - 1;
     const int local = ot - G.out0;
     const int i = local / mq, j = local % mq;
-    const SegI<R>* S = seg + G.item0;
+    const SegI<double>* S = seg + G.item0;
     const int nsq = G.nsq;
     // basis i rises on segment i and falls on segment i + 1 (same for j on wire q)
-    const SegI<R> a00 = S[i * nsq + j], a01 = S[i * nsq + j + 1], a10 = S[(i + 1) * nsq + j],
-                  a11 = S[(i + 1) * nsq + j + 1];
-    const cplx<R> vec = a00.rr + a01.rf + a10.fr + a11.ff;
-    auto IG = [](const SegI<R>& x) { return x.rr + x.rf + x.fr + x.ff; };
-    const cplx<R> sca = IG(a00) - IG(a01) - IG(a10) + IG(a11);
-    R f, sc, tpq;
-    if constexpr (sizeof(R) == 4) {
-      f = G.f;
-      sc = G.sc;
-      tpq = G.tpq;
-    } else {
-      f = G.fd;
-      sc = G.scd;
-      tpq = G.tpqd;
-    }
-    const cplx<R> z = mkc<R>(f * (tpq * vec.re - sc * sca.re), f * (tpq * vec.im - sc * sca.im));
-    const cplx<TV> zt = ccast<TV>(z);
-    Z[G.bpq + (int64_t)i * G.Kp + j] = zt;
-    Z[G.bqp + (int64_t)j * G.Kq + i] = zt;
+    const SegI<double> a00 = S[i * nsq + j], a01 = S[i * nsq + j + 1], a10 = S[(i + 1) * nsq + j],
+                       a11 = S[(i + 1) * nsq + j + 1];
+    const c128 vec = a00.rr + a01.rf + a10.fr + a11.ff;
+    auto IG = [](const SegI<double>& x) { return x.rr + x.rf + x.fr + x.ff; };
+    const c128 sca = IG(a00) - IG(a01) - IG(a10) + IG(a11);
+    const c128 z = mkc(G.f * (G.tpq * vec.re - G.sc * sca.re), G.f * (G.tpq * vec.im - G.sc * sca.im));
+    Z[G.bpq + (int64_t)i * G.Kp + j] = z;
+    Z[G.bqp + (int64_t)j * G.Kq + i] = z;
   }
 }
 
@@ -777,26 +745,22 @@ __global__ void __launch_bounds__(kFillF32Threads, 16) k_mutual_blocks_f32(
   }
 }
 
-template <typename R, typename TV>
-int launch_fill(swm_ctx* ctx, const GLTable& gl, unsigned long long* evals) {
-  const int ms = ctx->max_ns;
-  const int items_per_block = ms * ms;
-  // shared budget for segment pairs: 48 KB (float) or 64 KB (double)
-  const int cap_bytes = sizeof(R) == 4 ? 48 * 1024 : 64 * 1024;
-  int nbatch = std::max(1, cap_bytes / (int)(items_per_block * sizeof(SegI<R>)));
-  nbatch = std::min(nbatch, kFillThreads);
+int launch_fill_f64(swm_ctx* ctx, const GLTable& gl) {
+  if (ctx->nup <= 0) return SWM_OK;
+  const int items_per_block = ctx->max_ns * ctx->max_ns;
+  // blocks per CTA: at most what 32 KB hold, fewer where that leaves an SM without four CTAs
+  int nbatch = std::max(1, 32 * 1024 / (int)(items_per_block * sizeof(SegI<double>)));
+  nbatch = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nbatch, kFillThreads),
+                                                        ctx->nup / (4 * std::max(ctx->nsm, 1))));
   const size_t smem = round16(sizeof(BlockGeo) * nbatch) + 2 * round16(sizeof(int) * (nbatch + 1)) +
-                      sizeof(SegI<R>) * nbatch * items_per_block;
-  SWM_CK(allow_max_dyn_smem((const void*)k_mutual_blocks<R, TV>, ctx->smem_optin));
-  if (ctx->nup > 0) {
-    const int64_t grid = ceil_div(ctx->nup, nbatch);
-    ctx->prof_begin(SWM_K_FILL_MUTUAL);
-    k_mutual_blocks<R, TV><<<(unsigned)grid, kFillThreads, smem, ctx->stream>>>(
-        ctx->nup, ctx->ublk, ctx->col, ctx->bt, ctx->cx, ctx->cy, ctx->cz, ctx->tx, ctx->ty, ctx->tz, ctx->L, ctx->a,
-        ctx->ns, ctx->k, gl, ctx->full, nbatch, reinterpret_cast<cplx<TV>*>(ctx->Z), evals);
-    ctx->prof_end(SWM_K_FILL_MUTUAL);
-    SWM_LAUNCHED();
-  }
+                      sizeof(SegI<double>) * nbatch * items_per_block;
+  SWM_CK(allow_max_dyn_smem((const void*)k_mutual_blocks_f64, ctx->smem_optin));
+  ctx->prof_begin(SWM_K_FILL_MUTUAL);
+  k_mutual_blocks_f64<<<(unsigned)ceil_div(ctx->nup, nbatch), kFillThreads, smem, ctx->stream>>>(
+      ctx->nup, ctx->ublk, ctx->col, ctx->brow, ctx->bt, ctx->cx, ctx->cy, ctx->cz, ctx->tx, ctx->ty, ctx->tz, ctx->L,
+      ctx->a, ctx->ns, ctx->k, gl, ctx->full, nbatch, (c128*)ctx->Z, ctx->d_evals);
+  ctx->prof_end(SWM_K_FILL_MUTUAL);
+  SWM_LAUNCHED();
   return SWM_OK;
 }
 
@@ -815,7 +779,7 @@ int fill_self(swm_ctx* ctx, cudaStream_t s) {
   const int64_t nw = ctx->nw;
   int S = 2;
   while (S < ctx->max_ns) S <<= 1;
-  const unsigned grid_self = (unsigned)ceil_div(nw, kSelfThreads / S);
+  const unsigned grid_self = (unsigned)ceil_div(nw, kSelfThreads / ((ctx->prec == SWM_C128 ? 2 : 1) * S));
   ctx->prof_begin(SWM_K_FILL_SELF);
   if (ctx->prec == SWM_C128)
     k_self_blocks<double, double><<<grid_self, kSelfThreads, 0, s>>>(
@@ -832,7 +796,7 @@ int fill_self(swm_ctx* ctx, cudaStream_t s) {
 int fill_mutual(swm_ctx* ctx) {
   static const GLTable gl = make_gl();
   if (ctx->prec == SWM_C128) {
-    SWM_TRY((launch_fill<double, double>(ctx, gl, ctx->d_evals)));
+    SWM_TRY(launch_fill_f64(ctx, gl));
   } else if (ctx->nup > 0) {
     const int mm = ctx->max_ns - 1;
     const int acc_per_block = std::max(1, mm * mm);
