@@ -417,7 +417,7 @@ int swm_set_cloud(swm_ctx* ctx, int64_t nw, const double* centres, const double*
   ctx->built = ctx->solved = false;
   ctx->pattern_ok = false;
   ctx->rowwire = nullptr;
-  ctx->wrec = nullptr;
+  ctx->wrec = ctx->pkrec = ctx->pack = nullptr;
   ctx->nw = nw;
   auto& G = ctx->cloud_bufs;
   SWM_TRY(dalloc(ctx, G, (void**)&ctx->u_c, sizeof(double) * 3 * nw));
@@ -501,6 +501,7 @@ int swm_build(swm_ctx* ctx, double k, double r_c, int precision) {
   ctx->prec = precision == SWM_BF16 ? SWM_C64 : precision;
   ctx->bf16 = precision == SWM_BF16;
   ctx->E16 = nullptr;
+  ctx->pack = nullptr;
   if (!ctx->side) {  // the build's second stream (pattern column maps, self blocks, far-field data)
     SWM_CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
     SWM_CK(cudaEventCreateWithFlags(&ctx->side_ev[0], cudaEventDisableTiming));
@@ -511,7 +512,7 @@ int swm_build(swm_ctx* ctx, double k, double r_c, int precision) {
     dfree_group(ctx, ctx->pattern_bufs);
     ctx->pattern_ok = false;
     ctx->rowwire = nullptr;
-    ctx->wrec = nullptr;
+    ctx->wrec = ctx->pkrec = nullptr;
     ctx->uoff = nullptr;
     ctx->uoff_user = nullptr;
     SWM_TRY(build_pattern(ctx));

@@ -122,6 +122,8 @@ struct swm_ctx {
   int32_t* rowwire = nullptr;  // [N] internal wire of each scalar row
   void* wrec = nullptr;        // [nw] wire records of product form 75 in its order (built by the
                                // first solve that may use it after a pattern build)
+  void* pkrec = nullptr;       // [nw] wire records of product form 76 (product_pack.cu), with the pattern
+  void* pack = nullptr;        // E and the column map in that order, one record per wire, with the values
   void* rowinfo = nullptr;     // [N] row descriptors of E (value offset, column-map offset, length)
   int64_t nminv = 0;           // entries of the packed self-block inverses
   unsigned long long* d_evals = nullptr;  // fill evaluation counter (device)
@@ -303,6 +305,9 @@ void set_stateless_error(const std::string& msg);
 int gmres_solve(swm_ctx* ctx, double tol, int restart, int max_iter);
 int bicgstab_solve(swm_ctx* ctx, double tol, int max_iter);
 int build_wire_order(swm_ctx* ctx);
+// product_pack.cu: E as one record per wire for product form 76 (built by the first solve that uses it
+// after a build; krylov_common.cuh declares the product's launch)
+int ensure_pack(swm_ctx* ctx);
 // row descriptors of E (built once per build) and x = M^-1 y into ctx->Xv
 int ensure_rowinfo(swm_ctx* ctx);
 // y = y0 (ctx->guess, complex128) or 0 at the start of a solve, in the vector precision

@@ -2919,7 +2919,10 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
   // v = A u (active incidences) or, RS, v = b - A u (every incidence): u is its own gathered copy
   auto product = [&](cudaStream_t s, const c64* src, c64* dst, auto res_tag) -> int {
     constexpr bool RS = decltype(res_tag)::value;
-    SWM_TRY((launch_wm<c64, RS, true>(s, form, RS ? Pall : P, ctx, E, src, src, xst, dst, Bt, RQ, WBp)));
+    if (form == 76)
+      SWM_TRY(launch_pack(ctx, s, RS ? Pall : P, src, dst, Bt, xst, RS));
+    else
+      SWM_TRY((launch_wm<c64, RS, true>(s, form, RS ? Pall : P, ctx, E, src, src, xst, dst, Bt, RQ, WBp)));
     SWM_LAUNCHED();
     return SWM_OK;
   };
@@ -2928,17 +2931,18 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
     int found = 0;
     for (const auto& t : ctx->tuned)
       if (std::memcmp(t.shape, shape, sizeof(shape)) == 0) found = t.rb;
-    if (ctx->product_form >= 68 && ctx->product_form <= 75) {
+    if (ctx->product_form >= 68 && ctx->product_form <= 76) {
       form = ctx->product_form;
     } else if (found) {
       form = found;
     } else {
+      SWM_TRY(ensure_pack(ctx));
       // each shape once untimed and once timed on b (the product is idempotent)
       cudaEvent_t e0, e1;
       SWM_CK(cudaEventCreate(&e0));
       SWM_CK(cudaEventCreate(&e1));
       float best = 0.f;
-      for (int f : {68, 69, 70, 71, 72, 73, 74, 75}) {
+      for (int f : {68, 69, 70, 71, 72, 73, 74, 75, 76}) {
         form = f;
         SWM_TRY(product(st, Bt, Vv, std::true_type{}));
         SWM_CK(cudaEventRecord(e0, st));
@@ -2961,6 +2965,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       ctx->tuned.push_back(t);
     }
   }
+  if (form == 76) SWM_TRY(ensure_pack(ctx));
   ctx->stats.step_rhs_block = form;
   const unsigned gC = (unsigned)B.nchunk;
   auto launch_steps = [&](cudaStream_t s, int n) -> int {
@@ -3008,14 +3013,14 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
   if (use_graph) {
     struct Key {
       BmPtr B;
-      const void* ptr[11];
+      const void* ptr[13];
       Layout lay;
       int64_t bits;
     } gk;
     std::memset(&gk, 0, sizeof(gk));
     gk.B = B;
-    const void* ptrs[11] = {E, Y, Rv, Rh, Pv, Vv, Sv, Tv, Bt, ctx->off, ws->kst};
-    for (int i = 0; i < 11; ++i) gk.ptr[i] = ptrs[i];
+    const void* ptrs[13] = {E, Y, Rv, Rh, Pv, Vv, Sv, Tv, Bt, ctx->off, ws->kst, ctx->pack, ctx->pkrec};
+    for (int i = 0; i < 13; ++i) gk.ptr[i] = ptrs[i];
     gk.lay = ctx->offd;
     gk.bits = -(int64_t)(1000 + form);
     const unsigned char* kb = reinterpret_cast<const unsigned char*>(&gk);

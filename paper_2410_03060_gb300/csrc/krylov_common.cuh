@@ -94,6 +94,10 @@ struct ELoad<float, __nv_bfloat162> {
   }
 };
 
+// dst = src + E src for the pairs with an active incidence, or (res) Bv - (src + E src) for all, over
+// incidence-minor vectors [N][xst] (product form 76, product_pack.cu; after ensure_pack)
+int launch_pack(swm_ctx* ctx, cudaStream_t s, const KPtr& P, const c64* src, c64* dst, const c64* Bv, int xst, bool res);
+
 // Buffers of the persistent solve (persist.cu) handed over by the GMRES driver (krylov.cu).
 struct PSync {
   unsigned count;  // arrivals at grid barriers since the launch
