@@ -55,6 +55,31 @@ cudaError_t occupancy_cached(const void* fn, int threads, size_t smem, int* bloc
   return cudaSuccess;
 }
 
+static void give_back(swm_ctx* ctx, const Buf& b) {
+  if (ctx->user_free)
+    ctx->user_free(b.p, b.bytes, (void*)ctx->stream, ctx->user_arg);
+  else
+    cudaFreeAsync(b.p, ctx->stream);
+}
+
+bool release_spare(swm_ctx* ctx) {
+  bool any = !ctx->free_list.empty();
+  for (auto& b : ctx->free_list) give_back(ctx, b);
+  ctx->free_list.clear();
+  auto drop = [&](std::vector<Buf>& group, void** p) {
+    for (size_t i = 0; *p && i < group.size(); ++i)
+      if (group[i].p == *p) {
+        give_back(ctx, group[i]);
+        group.erase(group.begin() + i);
+        *p = nullptr;
+        any = true;
+      }
+  };
+  drop(ctx->build_bufs, &ctx->pack);
+  drop(ctx->pattern_bufs, &ctx->pkrec);
+  return any;
+}
+
 int dalloc(swm_ctx* ctx, std::vector<Buf>& group, void** out, size_t bytes) {
   bytes = std::max<size_t>((bytes + 255) / 256 * 256, 256);
   // reuse the smallest released buffer that fits without wasting more than half of it
@@ -72,9 +97,14 @@ int dalloc(swm_ctx* ctx, std::vector<Buf>& group, void** out, size_t bytes) {
   void* p = nullptr;
   if (ctx->user_alloc) {
     p = ctx->user_alloc(bytes, (void*)ctx->stream, ctx->user_arg);
+    if (!p && release_spare(ctx)) p = ctx->user_alloc(bytes, (void*)ctx->stream, ctx->user_arg);
     if (!p) return ctx->fail(SWM_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed");
   } else {
     cudaError_t e = cudaMallocAsync(&p, bytes, ctx->stream);
+    if (e == cudaErrorMemoryAllocation && release_spare(ctx)) {
+      cudaGetLastError();
+      e = cudaMallocAsync(&p, bytes, ctx->stream);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return ctx->fail(SWM_ENOMEM, "cudaMallocAsync(" + std::to_string(bytes) + "): " + cudaGetErrorString(e));
@@ -98,12 +128,7 @@ static void release_all(swm_ctx* ctx) {
   dfree_group(ctx, ctx->build_bufs);
   dfree_group(ctx, ctx->pattern_bufs);
   dfree_group(ctx, ctx->cloud_bufs);
-  for (auto& b : ctx->free_list) {
-    if (ctx->user_free)
-      ctx->user_free(b.p, b.bytes, (void*)ctx->stream, ctx->user_arg);
-    else
-      cudaFreeAsync(b.p, ctx->stream);
-  }
+  for (auto& b : ctx->free_list) give_back(ctx, b);
   ctx->free_list.clear();
 }
 
@@ -418,6 +443,7 @@ int swm_set_cloud(swm_ctx* ctx, int64_t nw, const double* centres, const double*
   ctx->pattern_ok = false;
   ctx->rowwire = nullptr;
   ctx->wrec = ctx->pkrec = ctx->pack = nullptr;
+  ctx->pack_refused = false;
   ctx->nw = nw;
   auto& G = ctx->cloud_bufs;
   SWM_TRY(dalloc(ctx, G, (void**)&ctx->u_c, sizeof(double) * 3 * nw));

@@ -124,6 +124,7 @@ struct swm_ctx {
                                // first solve that may use it after a pattern build)
   void* pkrec = nullptr;       // [nw] wire records of product form 76 (product_pack.cu), with the pattern
   void* pack = nullptr;        // E and the column map in that order, one record per wire, with the values
+  bool pack_refused = false;   // no memory was left for it (until the next cloud)
   void* rowinfo = nullptr;     // [N] row descriptors of E (value offset, column-map offset, length)
   int64_t nminv = 0;           // entries of the packed self-block inverses
   unsigned long long* d_evals = nullptr;  // fill evaluation counter (device)
@@ -235,6 +236,10 @@ namespace swm {
 
 // allocation helpers (api.cu)
 int dalloc(swm_ctx* ctx, std::vector<Buf>& group, void** out, size_t bytes);
+// Gives back, in stream order, what the context holds only to be faster: released buffers kept for reuse
+// and product form 76's copy of E (a solve that wants it makes it again).  False if there was nothing.
+// dalloc does so before it reports that an allocation failed.
+bool release_spare(swm_ctx* ctx);
 void dfree_group(swm_ctx* ctx, std::vector<Buf>& group);
 
 #define SWM_CK(call)                                                                 \
@@ -306,8 +311,9 @@ int gmres_solve(swm_ctx* ctx, double tol, int restart, int max_iter);
 int bicgstab_solve(swm_ctx* ctx, double tol, int max_iter);
 int build_wire_order(swm_ctx* ctx);
 // product_pack.cu: E as one record per wire for product form 76 (built by the first solve that uses it
-// after a build; krylov_common.cuh declares the product's launch)
-int ensure_pack(swm_ctx* ctx);
+// after a build; krylov_common.cuh declares the product's launch).  *ok = 0: E is too large for a second
+// copy, or no memory was left for it.
+int ensure_pack(swm_ctx* ctx, bool* ok);
 // row descriptors of E (built once per build) and x = M^-1 y into ctx->Xv
 int ensure_rowinfo(swm_ctx* ctx);
 // y = y0 (ctx->guess, complex128) or 0 at the start of a solve, in the vector precision

@@ -2936,13 +2936,15 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
     } else if (found) {
       form = found;
     } else {
-      SWM_TRY(ensure_pack(ctx));
+      bool packed = false;
+      SWM_TRY(ensure_pack(ctx, &packed));
       // each shape once untimed and once timed on b (the product is idempotent)
       cudaEvent_t e0, e1;
       SWM_CK(cudaEventCreate(&e0));
       SWM_CK(cudaEventCreate(&e1));
       float best = 0.f;
       for (int f : {68, 69, 70, 71, 72, 73, 74, 75, 76}) {
+        if (f == 76 && !packed) continue;
         form = f;
         SWM_TRY(product(st, Bt, Vv, std::true_type{}));
         SWM_CK(cudaEventRecord(e0, st));
@@ -2965,7 +2967,11 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       ctx->tuned.push_back(t);
     }
   }
-  if (form == 76) SWM_TRY(ensure_pack(ctx));
+  if (form == 76) {  // without its copy of E: form 75, the same sums from E itself
+    bool packed = false;
+    SWM_TRY(ensure_pack(ctx, &packed));
+    if (!packed) form = 75;
+  }
   ctx->stats.step_rhs_block = form;
   const unsigned gC = (unsigned)B.nchunk;
   auto launch_steps = [&](cudaStream_t s, int n) -> int {

@@ -324,36 +324,64 @@ int pack_rq(int np) {
 
 }  // namespace
 
-int ensure_pack(swm_ctx* ctx) {
+// The copy's bytes at most: column maps rounded up to 16 bytes, one padding column and one padding row of
+// entries per wire.
+static size_t pack_most(const swm_ctx* ctx) {
+  return std::max<size_t>((size_t)4 * ctx->offd.ncm + (size_t)(20 + 8 * (kMaxM + 1)) * ctx->nw +
+                              (size_t)8 * (ctx->offd.nval + ctx->offd.ncm),
+                          16);
+}
+
+// Only a second copy of an E that leaves the memory mostly free: up to a ninth of the card (a million
+// wires take 5 GB).  Larger systems keep form 75, which reads E where it lies.
+constexpr size_t kPackMost = (size_t)32 << 30;
+
+static int make_pack(swm_ctx* ctx) {
   const int64_t nw = ctx->nw;
   SWM_CK(allow_max_dyn_smem((const void*)k_spmv_pack<true>, ctx->smem_optin));
   SWM_CK(allow_max_dyn_smem((const void*)k_spmv_pack<false>, ctx->smem_optin));
   if (!ctx->pkrec) {
     std::vector<Buf> tmp;
+    void* recs = nullptr;
     int64_t *bytes = nullptr, *at = nullptr;
-    SWM_TRY(dalloc(ctx, ctx->pattern_bufs, &ctx->pkrec, sizeof(PackRec) * nw));
-    SWM_TRY(dalloc(ctx, tmp, (void**)&bytes, sizeof(int64_t) * nw));
-    SWM_TRY(dalloc(ctx, tmp, (void**)&at, sizeof(int64_t) * (nw + 1)));
-    PackRec* rec = reinterpret_cast<PackRec*>(ctx->pkrec);
-    k_pack_order<<<(unsigned)ceil_div(nw, kPackWin), 1024, 0, ctx->stream>>>(nw, ctx->offd, ctx->off, rec, bytes);
-    SWM_LAUNCHED();
-    const void* in[1] = {bytes};
-    const int is64[1] = {1};
-    int64_t* out[1] = {at};
-    SWM_TRY(exclusive_scan_multi(ctx, 1, in, is64, out, nw));
-    k_pack_place<<<(unsigned)ceil_div(nw, 256), 256, 0, ctx->stream>>>(nw, at, rec);
-    SWM_LAUNCHED();
+    int rc = dalloc(ctx, ctx->pattern_bufs, &recs, sizeof(PackRec) * nw);
+    if (rc >= 0) rc = dalloc(ctx, tmp, (void**)&bytes, sizeof(int64_t) * nw);
+    if (rc >= 0) rc = dalloc(ctx, tmp, (void**)&at, sizeof(int64_t) * (nw + 1));
+    if (rc >= 0) {
+      PackRec* rec = reinterpret_cast<PackRec*>(recs);
+      k_pack_order<<<(unsigned)ceil_div(nw, kPackWin), 1024, 0, ctx->stream>>>(nw, ctx->offd, ctx->off, rec, bytes);
+      SWM_LAUNCHED();
+      const void* in[1] = {bytes};
+      const int is64[1] = {1};
+      int64_t* out[1] = {at};
+      rc = exclusive_scan_multi(ctx, 1, in, is64, out, nw);
+      if (rc >= 0) {
+        k_pack_place<<<(unsigned)ceil_div(nw, 256), 256, 0, ctx->stream>>>(nw, at, rec);
+        SWM_LAUNCHED();
+        ctx->pkrec = recs;
+      }
+    }
     dfree_group(ctx, tmp);
+    if (rc < 0) return rc;
   }
   if (!ctx->pack) {
-    // at most: column maps rounded up to 16 bytes, one padding column and one padding row of entries per wire
-    const size_t most = (size_t)4 * ctx->offd.ncm + (size_t)(20 + 8 * (kMaxM + 1)) * nw +
-                        (size_t)8 * (ctx->offd.nval + ctx->offd.ncm);
-    SWM_TRY(dalloc(ctx, ctx->build_bufs, &ctx->pack, std::max<size_t>(most, 16)));
+    SWM_TRY(dalloc(ctx, ctx->build_bufs, &ctx->pack, pack_most(ctx)));
+    if (!ctx->pkrec) return SWM_ENOMEM;  // given back to make room
     k_pack_fill<<<(unsigned)ceil_div(nw * 32, 256), 256, 0, ctx->stream>>>(
         nw, reinterpret_cast<const PackRec*>(ctx->pkrec), ctx->offd, (const c64*)ctx->Zp, (unsigned char*)ctx->pack);
     SWM_LAUNCHED();
   }
+  return SWM_OK;
+}
+
+int ensure_pack(swm_ctx* ctx, bool* ok) {
+  *ok = pack_most(ctx) <= kPackMost && !ctx->pack_refused;
+  if (!*ok) return SWM_OK;
+  const int rc = make_pack(ctx);
+  if (rc != SWM_ENOMEM) return rc;
+  release_spare(ctx);
+  ctx->pack_refused = true;
+  *ok = false;
   return SWM_OK;
 }
 
