@@ -150,11 +150,92 @@ __global__ void __launch_bounds__(128) k_invert_self(int64_t nw, const int32_t* 
   }
 }
 
-// E_pq = Z_pq Minv_q for every kept block with q != p; one warp per block.
-template <typename TV>
-__global__ void k_form_E(int64_t nb, const int32_t* __restrict__ col, const int64_t* __restrict__ bt,
-                         const int32_t* __restrict__ m, Layout full, Layout offd, const cplx<TV>* __restrict__ Z,
-                         const int64_t* __restrict__ moff, const cplx<TV>* __restrict__ Minv, cplx<TV>* __restrict__ E) {
+// E_pq = Z_pq Minv_q for every kept block with p != q, complex64.  A warp takes `per` consecutive blocks (q, p) of the
+// rows q (up to 32), a lane a column of one of them: Z is symmetric bit for bit (Z_pq = Z_qp^T, stored twice by the
+// fill), so row i of Z_pq is column i of Z_qp, and the lanes of a warp read Z along the rows of q
+// (consecutive blocks are consecutive columns) and share the entries of Minv_q, each entry read once for
+// the whole row of E_pq.  Bound by HBM in float32.  A warp per block with a lane per entry read every
+// entry of Z and Minv_q m_q times and divided for its indices: 1,000,000 wires 4.14 -> 1.81 ms, entire
+// coupling of 1,000 wires 0.49 -> 0.25 ms.
+constexpr int kFormThreads = 128;
+struct FormBlk {
+  int64_t z, e, mi;  // first value of Z_qp, of E_pq, of Minv_q
+  int Kz, Ke, mq;
+};
+__global__ void __launch_bounds__(kFormThreads) k_form_E(int64_t nb, const int32_t* __restrict__ col,
+                                                         const int64_t* __restrict__ bt, const int32_t* __restrict__ m,
+                                                         Layout full, Layout offd, const c64* __restrict__ Z,
+                                                         const int64_t* __restrict__ moff,
+                                                         const c64* __restrict__ Minv, c64* __restrict__ E, int per) {
+  __shared__ FormBlk sb[kFormThreads / 32][32];
+  __shared__ int sp[kFormThreads / 32][33];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int64_t b0 = (blockIdx.x * (int64_t)(kFormThreads / 32) + wp) * per;
+  if (b0 >= nb) return;
+  FormBlk* B = sb[wp];
+  int* pre = sp[wp];
+  int mp = 0, mq = 0;
+  if (lane < per && b0 + lane < nb) {
+    const int64_t b = b0 + lane, t = bt[b];
+    const int p = col[b], q = col[t];
+    if (p != q) {
+      mp = m[p];
+      mq = m[q];
+      FormBlk f;
+      f.z = full.rowbase[q] + full.colpos[b];
+      f.Kz = full.K[q];
+      f.e = offd.rowbase[p] + offd.colpos[t];
+      f.Ke = offd.K[p];
+      f.mi = moff[q];
+      f.mq = mq;
+      B[lane] = f;
+    }
+  }
+  int inc = mp;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += o;
+  }
+  pre[lane + 1] = inc;
+  if (lane == 0) pre[0] = 0;
+  const int mmax = __reduce_max_sync(0xffffffffu, mq);
+  __syncwarp();
+  const int total = pre[32];
+  for (int t = lane; t < total; t += 32) {
+    int lo = 0;  // the last block with pre[lo] <= t: one with columns
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+      if (pre[lo + d] <= t) lo += d;
+    const FormBlk f = B[lo];
+    const int i = t - pre[lo];
+    const c64* z = Z + f.z + i;
+    const c64* Mi = Minv + f.mi;
+    c64* e = E + f.e + (int64_t)i * f.Ke;
+    for (int j0 = 0; j0 < mmax; j0 += 8) {
+      c64 acc[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] = mkc<float>(0, 0);
+      for (int l = 0; l < f.mq; ++l) {
+        const c64 zl = z[(int64_t)l * f.Kz];
+        const c64* ml = Mi + l * f.mq + j0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (j0 + j < f.mq) cfma(acc[j], zl, ml[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j0 + j < f.mq) e[j0 + j] = acc[j];
+    }
+  }
+}
+
+// The same, one warp per block and a lane per entry: the float64 form.  There the multiply-adds issue
+// sixteen times slower than the loads they wait for, and a lane per column spends more of them on lanes
+// past the row and column counts of its own block (10,007 wires: 118 us here, 182 us by columns).
+__global__ void k_form_E_entries(int64_t nb, const int32_t* __restrict__ col, const int64_t* __restrict__ bt,
+                         const int32_t* __restrict__ m, Layout full, Layout offd, const c128* __restrict__ Z,
+                         const int64_t* __restrict__ moff, const c128* __restrict__ Minv, c128* __restrict__ E) {
   const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (b >= nb) return;
@@ -165,10 +246,10 @@ __global__ void k_form_E(int64_t nb, const int32_t* __restrict__ col, const int6
   const int Kf = full.K[p], Ko = offd.K[p];
   const int64_t zb = full.rowbase[p] + full.colpos[b];
   const int64_t eb = offd.rowbase[p] + offd.colpos[b];
-  const cplx<TV>* Mi = Minv + moff[q];
+  const c128* Mi = Minv + moff[q];
   for (int e = lane; e < mp * mq; e += 32) {
     const int i = e / mq, j = e % mq;
-    cplx<TV> acc = mkc<TV>(0, 0);
+    c128 acc = mkc(0.0, 0.0);
     for (int l = 0; l < mq; ++l) cfma(acc, Z[zb + (int64_t)i * Kf + l], Mi[l * mq + j]);
     E[eb + (int64_t)i * Ko + j] = acc;
   }
@@ -204,16 +285,20 @@ int precond_invert(swm_ctx* ctx, cudaStream_t s) {
 
 // E = Z M^-1 off the diagonal, on the context's stream (after the fill and the inversion).
 int precond_form_E(swm_ctx* ctx) {
-  const unsigned g2 = (unsigned)std::max<int64_t>(1, ceil_div(ctx->nb * 32, 256));
+  const unsigned g1 = (unsigned)std::max<int64_t>(1, ceil_div(ctx->nb * 32, 256));
+  // 32 blocks per warp, fewer (down to 4, one pass over their columns) while that leaves warps to spare
+  int per = 32;
+  while (per > 4 && ctx->nb < (int64_t)per * 16 * std::max(ctx->nsm, 1)) per >>= 1;
+  const unsigned g2 = (unsigned)std::max<int64_t>(1, ceil_div(ctx->nb, (int64_t)per * (kFormThreads / 32)));
   ctx->prof_begin(SWM_K_FORM_E);
   if (ctx->prec == SWM_C128)
-    k_form_E<double><<<g2, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
+    k_form_E_entries<<<g1, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
                                                   (const c128*)ctx->Z, ctx->minv_off, (const c128*)ctx->Minv,
                                                   (c128*)ctx->Zp);
   else
-    k_form_E<float><<<g2, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
+    k_form_E<<<g2, kFormThreads, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
                                                  (const c64*)ctx->Z, ctx->minv_off, (const c64*)ctx->Minv,
-                                                 (c64*)ctx->Zp);
+                                                 (c64*)ctx->Zp, per);
   ctx->prof_end(SWM_K_FORM_E);
   SWM_LAUNCHED();
   return SWM_OK;
