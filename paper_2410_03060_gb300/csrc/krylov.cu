@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256, MINB) k_spmv_w(KPtr P, const int64_t* __r
   const int64_t p0 = (int64_t)blockIdx.x * WB;
   const int r0 = blockIdx.y * RG;
   const int pl = (int)threadIdx.x / RG, rl = (int)threadIdx.x % RG;
-  const int64_t p = p0 + pl;
+  int64_t p = p0 + pl;
   const int r = r0 + rl;
   if (pl >= WB || p >= nw || r >= P.R || !(ALL || P.active[r])) return;
   const int64_t op = off[p];
@@ -1047,7 +1047,7 @@ __device__ void step_arrive(const KPtr& P, int j, bool closing) {
 // and the residual test, and, unless this is the closing pass or r stopped, forms the first-pass
 // coefficients of column j and the coefficients of the update pass.
 template <typename TV>
-__device__ void dots_tail(const KPtr& P, int j, int r, bool closing) {
+__device__ void dots_tail(const KPtr& P, int j, int r, bool closing, const c128* __restrict__ part, int np) {
   const int R1 = P.restart + 1, RS = P.restart;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   __shared__ c128 sv[SWM_MAX_RESTART + 1], tv[SWM_MAX_RESTART + 1], col[SWM_MAX_RESTART + 1];
@@ -1055,10 +1055,9 @@ __device__ void dots_tail(const KPtr& P, int j, int r, bool closing) {
   __shared__ c128 ssn[SWM_MAX_RESTART];
   __shared__ double rho_s;
   __shared__ int go_on;
-  const c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
   for (int i = wp; i < 2 * (j + 1); i += kRows / 32) {
     if (closing && (i & 1)) continue;
-    const c128 v = sum_partials_c(part + (int64_t)i * P.nchunk, 1, P.nchunk, lane);
+    const c128 v = sum_partials_c(part + (int64_t)i * np, 1, np, lane);
     if (lane == 0) {
       if (i & 1)
         tv[i >> 1] = v;
@@ -1104,16 +1103,18 @@ __device__ void dots_tail(const KPtr& P, int j, int r, bool closing) {
       }
       // new rotation zeroing the subdiagonal rho (real, >= 0)
       const c128 a = col[l];
-      const double aa = sqrt(a.re * a.re + a.im * a.im);
-      const double nu = sqrt(aa * aa + rho * rho);
+      const double a2 = a.re * a.re + a.im * a.im;
       double c;
       c128 sg;
-      if (aa == 0.0) {
+      if (a2 == 0.0) {
         c = 0.0;
         sg = mkc(1.0, 0.0);
       } else {
-        c = aa / nu;
-        sg = mkc(a.re / aa * rho / nu, a.im / aa * rho / nu);
+        // two reciprocal roots in place of two roots and five divisions, on the one serial chain of a step
+        const double ra = rsqrt(a2), rnu = rsqrt(fma(rho, rho, a2));
+        c = a2 * ra * rnu;
+        const double f = ra * (rho * rnu);
+        sg = mkc(a.re * f, a.im * f);
       }
       P.cs[(int64_t)r * RS + l] = c;
       P.sn[(int64_t)r * RS + l] = sg;
@@ -1177,15 +1178,41 @@ __device__ void dots_tail(const KPtr& P, int j, int r, bool closing) {
   if (threadIdx.x == 0) step_arrive(P, j, closing);
 }
 
+// Sums over the warp of eight values: lanes 4 i .. 4 i + 3 return that of v[i].  Each of the first three
+// exchanges halves the number of values a lane carries (9 additions for 8 sums; one sum after the other
+// takes 40, which in float64 cost half as much as reading the rows).
+template <typename TV>
+__device__ __forceinline__ TV warp_sum8(const TV (&v)[8], int lane) {
+  const bool h = lane & 16, m = lane & 8, l = lane & 4;
+  TV p[4], q[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[i] = (h ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h ? v[i] : v[i + 4], 16);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) q[i] = (m ? p[i + 2] : p[i]) + __shfl_xor_sync(0xffffffffu, m ? p[i] : p[i + 2], 8);
+  TV k = (l ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, l ? q[0] : q[1], 4);
+  k += __shfl_xor_sync(0xffffffffu, k, 2);
+  return k + __shfl_xor_sync(0xffffffffu, k, 1);
+}
+
+constexpr int kDotsGroup = 32;  // chunks whose partial sums one CTA adds before the last CTA does
+template <typename TV>
+constexpr int kDotsRows = sizeof(TV) == 4 ? 8 : 4;  // rows of u and w in a lane's registers
+
 // Dots of step j, one CTA per chunk of rows and right-hand side: for i < j the pairs
 // (q_i^H u, q_i^H w), and (|u|^2, u^H w), where u is the pending vector and w = A u; the closing
-// pass of a cycle (j = jmax, no product) takes only the first of each pair.  The chunk's rows of u
-// and w are staged in shared memory; the warps take (i, row slice) items, q_j standing for u itself,
-// with the rows split into S slices while j + 1 < 8 so that every warp streams, and eight loads in
-// flight per lane.  Slice sums are added in a fixed order (results do not depend on timing).
-template <typename TV, typename TQ = cplx<TV>>
-__global__ void __launch_bounds__(kRows) k_dots(KPtr P, const cplx<TV>* __restrict__ U,
-                                                const cplx<TV>* __restrict__ Wv, const TQ* __restrict__ V) {
+// pass of a cycle (j = jmax, no product) takes only the first of each pair.  Bound by HBM (the basis is
+// read once; in float64 by its multiply-adds).  A lane keeps its rows of u and w in registers and every
+// warp passes over all the basis vectors, the next one's loads in flight while one is summed, so the warps
+// stay balanced at every j and nothing waits for a staged copy.  The partial sums of kDotsGroup chunks are
+// added by the group's last CTA, those of the groups by the last CTA of all: a single CTA adding 1,003
+// partials of each of up to 100 sums took as long as the pass over the rows.  The rows of a warp (256) are
+// added in float32 as a tree, depth 13 (64 in sequence before), the rest in float64.  Every sum has a fixed
+// order (results do not depend on timing).  400,001 wires at one incidence, 37 steps: 5.6 ->
+// 3.7 ms; 24,535 wires at 181 incidences 2.6 -> 2.0 ms.
+template <typename TV, typename TQ>
+__global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __restrict__ U,
+                                                                         const cplx<TV>* __restrict__ Wv,
+                                                                         const TQ* __restrict__ V) {
   if (P.st->cycle_done) return;
   const int j = P.st->j, r = blockIdx.y;
   const bool closing = j >= P.st->jmax;
@@ -1194,83 +1221,127 @@ __global__ void __launch_bounds__(kRows) k_dots(KPtr P, const cplx<TV>* __restri
     return;
   }
   const int R1 = P.restart + 1;
+  constexpr int kWarps = kRows / 32, KR = kDotsRows<TV>;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const int64_t n0 = (int64_t)blockIdx.x * P.chunk;
-  const int cnt = (int)min((int64_t)P.chunk, P.N - n0);
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  cplx<TV>* u_sm = reinterpret_cast<cplx<TV>*>(sm_raw);  // [chunk]
-  cplx<TV>* w_sm = u_sm + P.chunk;                       // [chunk]
-  __shared__ c128 slot[2 * (SWM_MAX_RESTART + 1)];
-  const cplx<TV>* u = U + (int64_t)r * P.N + n0;
-  const cplx<TV>* w = Wv + (int64_t)r * P.N + n0;
-  for (int t = threadIdx.x; t < cnt; t += kRows) {
-    u_sm[t] = u[t];
-    if (!closing) w_sm[t] = w[t];
-  }
-  __syncthreads();
-  constexpr int kWarps = kRows / 32;
-  const int S = j + 1 >= kWarps ? 1 : kWarps / (j + 1);  // row slices per i
-  const int len = ((cnt + S - 1) / S + 31) / 32 * 32;
-  for (int item = wp; item < (j + 1) * S; item += kWarps) {
-    const int i = item / S, sl = item % S;
-    const int lo = sl * len, hi = min(cnt, lo + len);
-    // q_i from the basis, or (i == j) the pending vector u itself from shared memory; a basis in
-    // the vector type is read through one pointer, a half-precision one converted on load
-    constexpr bool full = std::is_same<TQ, cplx<TV>>::value;
-    const TQ* vq = V + ((int64_t)i * P.R + r) * P.N + n0;  // i <= j <= restart: inside the basis
-    const cplx<TV>* vi = full ? (i < j ? reinterpret_cast<const cplx<TV>*>(vq) : u_sm) : u_sm;
-    const bool own = i >= j;
-    const float qsi = P.qsi;
-    auto ldv = [&](int t) -> cplx<TV> {
-      if constexpr (full) return vi[t];
-      else return own ? u_sm[t] : QStore<TV, TQ>::ld(vq + t, qsi);
+  double* slot = reinterpret_cast<double*>(sm_raw);  // [j + 1][kWarps][4]
+  const int64_t end = min(P.N, (int64_t)(blockIdx.x + 1) * P.chunk);
+  const int64_t rn = (int64_t)r * P.N, vst = (int64_t)P.R * P.N;
+  const float qsi = P.qsi;
+  bool first = true;
+  for (int64_t n0 = (int64_t)blockIdx.x * P.chunk; n0 < end; n0 += KR * kRows, first = false) {
+    const int64_t n = n0 + threadIdx.x;
+    const int left = n < end ? (int)min((int64_t)KR, (end - n + kRows - 1) / kRows) : 0;  // rows of this thread
+    cplx<TV> x[KR], y[KR];
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+      x[k] = y[k] = mkc<TV>(0, 0);
+      if (k < left) {
+        x[k] = U[rn + n + kRows * k];
+        if (!closing) y[k] = Wv[rn + n + kRows * k];
+      }
+    }
+    const TQ* vq = V + rn + n;
+    auto load = [&](cplx<TV> (&v)[KR]) {
+#pragma unroll
+      for (int k = 0; k < KR; ++k) v[k] = k < left ? QStore<TV, TQ>::ld(vq + kRows * k, qsi) : mkc<TV>(0, 0);
+      vq += vst;
     };
-    cplx<TV> a = mkc<TV>(0, 0), b = mkc<TV>(0, 0);
-    int t = lo + lane;
-    for (; t + 224 < hi; t += 256) {
-      cplx<TV> v[8];
+    auto dot = [&](const cplx<TV> (&v)[KR], TV* o) {
+      cplx<TV> a = mkc<TV>(0, 0), b = mkc<TV>(0, 0);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = ldv(t + 32 * k);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const cplx<TV> x = u_sm[t + 32 * k];
-        a.re = fma(v[k].re, x.re, fma(v[k].im, x.im, a.re));
-        a.im = fma(v[k].re, x.im, fma(-v[k].im, x.re, a.im));
-        if (!closing) {
-          const cplx<TV> y = w_sm[t + 32 * k];
-          b.re = fma(v[k].re, y.re, fma(v[k].im, y.im, b.re));
-          b.im = fma(v[k].re, y.im, fma(-v[k].im, y.re, b.im));
-        }
+      for (int k = 0; k < KR; ++k) {
+        a.re = fma(v[k].re, x[k].re, fma(v[k].im, x[k].im, a.re));
+        a.im = fma(v[k].re, x[k].im, fma(-v[k].im, x[k].re, a.im));
+        b.re = fma(v[k].re, y[k].re, fma(v[k].im, y[k].im, b.re));
+        b.im = fma(v[k].re, y[k].im, fma(-v[k].im, y[k].re, b.im));
       }
-    }
-    for (; t < hi; t += 32) {
-      const cplx<TV> v = ldv(t), x = u_sm[t];
-      a.re = fma(v.re, x.re, fma(v.im, x.im, a.re));
-      a.im = fma(v.re, x.im, fma(-v.im, x.re, a.im));
-      if (!closing) {
-        const cplx<TV> y = w_sm[t];
-        b.re = fma(v.re, y.re, fma(v.im, y.im, b.re));
-        b.im = fma(v.re, y.im, fma(-v.im, y.re, b.im));
+      o[0] = a.re;
+      o[1] = a.im;
+      o[2] = b.re;
+      o[3] = b.im;
+    };
+    cplx<TV> v0[KR], v1[KR];
+    if (j > 0) load(v0);
+    for (int i = 0; i <= j; i += 2) {  // the j-th vector is u itself
+      TV d[8];
+      if (i + 1 < j) load(v1);
+      if (i < j)
+        dot(v0, d);
+      else
+        dot(x, d);
+      if (i + 2 < j) load(v0);
+      if (i + 1 < j)
+        dot(v1, d + 4);
+      else if (i + 1 == j)
+        dot(x, d + 4);
+      else
+        d[4] = d[5] = d[6] = d[7] = TV(0);
+      const double t = (double)warp_sum8<TV>(d, lane);
+      const int ii = i + (lane >> 4);
+      if ((lane & 3) == 0 && ii <= j) {
+        double* s = slot + (ii * kWarps + wp) * 4 + ((lane >> 2) & 3);  // this lane's own over all the pieces
+        *s = first ? t : *s + t;
       }
-    }
-    const double ar = warp_sum((double)a.re), ai = warp_sum((double)a.im);
-    const double br = warp_sum((double)b.re), bi = warp_sum((double)b.im);
-    if (lane == 0) {
-      slot[2 * item] = mkc(ar, ai);
-      slot[2 * item + 1] = mkc(br, bi);
     }
   }
   __syncthreads();
-  // partials laid out [r][2 i + k][chunk]: the last CTA reads each as one contiguous run
+  // partials laid out [r][2 i + k][chunk]: a group of chunks is one contiguous run
   c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
   for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
-    const int i = e >> 1, k = e & 1;
-    c128 v = slot[2 * (i * S) + k];
-    for (int sl = 1; sl < S; ++sl) v = v + slot[2 * (i * S + sl) + k];
-    part[(int64_t)e * P.nchunk + blockIdx.x] = v;
+    const double* sl = slot + (e >> 1) * (kWarps * 4) + 2 * (e & 1);
+    c128 t = mkc(0.0, 0.0);
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) t = t + mkc(sl[4 * w], sl[4 * w + 1]);
+    part[(int64_t)e * P.nchunk + blockIdx.x] = t;
   }
-  if (!last_cta(P, r)) return;
-  dots_tail<TV>(P, j, r, closing);
+  if (P.ngroup <= 1) {
+    if (!last_cta(P, r)) return;
+    dots_tail<TV>(P, j, r, closing, part, P.nchunk);
+    return;
+  }
+  // the last CTA of the group adds the group's partials, then the last group's CTA goes on
+  __shared__ bool last;
+  const int gr = blockIdx.x / kDotsGroup;
+  const int c0 = gr * kDotsGroup, gn = min(kDotsGroup, P.nchunk - c0);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned* cnt = P.gcounter + (int64_t)r * P.ngroup + gr;
+    last = atomicAdd(cnt, 1u) == (unsigned)gn - 1;
+    if (last) *cnt = 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  c128* gpart = P.gpart + (int64_t)r * 2 * R1 * P.ngroup;
+  constexpr int EB = 4;  // sums of a warp whose loads are in flight together
+  for (int e0 = wp; e0 < 2 * (j + 1); e0 += EB * kWarps) {
+    double2 v[EB];
+#pragma unroll
+    for (int u = 0; u < EB; ++u) {
+      const int e = e0 + u * kWarps;
+      v[u] = make_double2(0.0, 0.0);
+      if (e < 2 * (j + 1) && lane < gn)
+        v[u] = __ldcg(reinterpret_cast<const double2*>(part + (int64_t)e * P.nchunk + c0 + lane));
+    }
+#pragma unroll
+    for (int u = 0; u < EB; u += 4) {
+      const double d[8] = {v[u].x,     v[u].y,     v[u + 1].x, v[u + 1].y,
+                           v[u + 2].x, v[u + 2].y, v[u + 3].x, v[u + 3].y};
+      const double t = warp_sum8<double>(d, lane);
+      const int e = e0 + (u + (lane >> 3)) * kWarps;
+      if ((lane & 3) == 0 && e < 2 * (j + 1))
+        reinterpret_cast<double*>(gpart + (int64_t)e * P.ngroup + gr)[(lane >> 2) & 1] = t;
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&P.counter[r], 1u) == (unsigned)P.ngroup - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  dots_tail<TV>(P, j, r, closing, gpart, P.ngroup);
 }
 
 // Update of step j (after its dots): q_j = (u - Q s) / rho goes to V_j and the next pending vector
@@ -1518,14 +1589,21 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   P.max_iter = max_iter;
   P.qs = kFullBasis ? 1.f : (float)std::sqrt((double)std::max<int64_t>(1, N));
   P.qsi = 1.f / P.qs;
-  // rows per CTA of the Gram-Schmidt kernels, at least kRows and at most kMaxChunk (the dots stage
-  // a chunk of u and w in shared memory): the update about 16 CTAs per SM over all right-hand
-  // sides; the dots about 4, so that the last CTA of each right-hand side adds fewer partial sums
+  // rows per CTA of the Gram-Schmidt kernels: the update about 16 CTAs per SM over all right-hand
+  // sides, at most kMaxChunk; the dots one wave of CTAs (fewest partial sums), or, where that would leave
+  // a right-hand side fewer than 16 CTAs, up to four pieces per CTA in several waves; in float64 one piece
+  // per CTA (adding the next piece's sums would cost float64 instructions, which set the time there)
   const int64_t nsm = std::max(ctx->nsm, 1);
   P.uchunk = (int)std::min<int64_t>(kMaxChunk, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, 16 * nsm), kRows) * kRows));
   P.nuchunk = (int)ceil_div(N, P.uchunk);
-  P.chunk = (int)std::min<int64_t>(kMaxChunk, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, 4 * nsm), kRows) * kRows));
+  constexpr int64_t dpiece = kDotsRows<TV> * kRows;
+  const int64_t slots = 2 * nsm;
+  int64_t dchunk = ceil_div(N, std::max<int64_t>(1, slots / R));
+  if (sizeof(TV) == 8) dchunk = std::min(dchunk, dpiece);
+  if (slots / R < 16) dchunk = std::min(dchunk, 4 * dpiece);
+  P.chunk = (int)(ceil_div(std::max<int64_t>(dchunk, kRows), 32) * 32);
   P.nchunk = (int)ceil_div(N, P.chunk);
+  P.ngroup = P.nchunk > 2 * kDotsGroup ? (int)ceil_div(P.nchunk, kDotsGroup) : 1;
   const int R1 = restart + 1;
   // The workspace persists across solves of the same size, so buffer addresses (and the captured
   // graph that bakes them in) stay the same from one solve to the next.
@@ -1570,6 +1648,8 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
     SWM_TRY(dalloc(ctx, K, (void**)&P.gam, sizeof(c128) * R));
     SWM_TRY(dalloc(ctx, K, (void**)&P.coef, sizeof(c128) * R * restart));
     SWM_TRY(dalloc(ctx, K, (void**)&P.part, sizeof(c128) * (size_t)R * P.nchunk * 2 * R1));
+    SWM_TRY(dalloc(ctx, K, (void**)&P.gpart, sizeof(c128) * (size_t)R * P.ngroup * 2 * R1));
+    SWM_TRY(dalloc(ctx, K, (void**)&P.gcounter, sizeof(unsigned) * (size_t)R * P.ngroup));
     SWM_TRY(dalloc(ctx, K, (void**)&P.partn, sizeof(double) * (size_t)R * P.nchunk));
     SWM_TRY(dalloc(ctx, K, (void**)&ws->Y, sizeof(cplx<TV>) * R * N));
     SWM_TRY(dalloc(ctx, K, (void**)&ws->W0, sizeof(cplx<TV>) * R * N));
@@ -1621,6 +1701,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   if (!persisted) {
     SWM_CK(cudaMemsetAsync(P.st, 0, sizeof(KState), st));
     SWM_CK(cudaMemsetAsync(P.counter, 0, sizeof(unsigned) * (R + 1), st));
+    SWM_CK(cudaMemsetAsync(P.gcounter, 0, sizeof(unsigned) * (size_t)R * P.ngroup, st));
     if (!given_b) SWM_CK(cudaMemsetAsync(Y, 0, sizeof(cplx<TV>) * R * N, st));
   }
   const dim3 g_chunk((unsigned)P.nchunk, R), g_uchunk((unsigned)P.nuchunk, R);
@@ -1746,8 +1827,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
       SWM_TRY(allow_wm<TE>(ctx));
     }
   }
-  const size_t dots_smem = 2 * sizeof(cplx<TV>) * (size_t)P.chunk;
-  if (dots_smem > 48 * 1024) SWM_CK(allow_max_dyn_smem((const void*)k_dots<TV, TQ>, ctx->smem_optin));
+  const size_t dots_smem = sizeof(double) * 4 * (kRows / 32) * (size_t)R1;  // at most 33 KB
   // back substitution stages the triangle in shared memory when it fits
   size_t bs_smem = sizeof(c128) * (size_t)restart * restart;
   if (bs_smem > 160 * 1024) bs_smem = 0;

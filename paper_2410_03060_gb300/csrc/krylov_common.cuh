@@ -40,7 +40,10 @@ struct KPtr {
   c128* gam;          // [R]
   c128* coef;         // [R][restart]
   c128* part;         // [R][2 (restart + 1)][nchunk]
+  c128* gpart;        // [R][2 (restart + 1)][ngroup]: sums over the groups of chunks
+  unsigned* gcounter; // [R][ngroup] CTAs of the current pass that have arrived
   double* partn;      // [R][nchunk]
+  int ngroup;         // groups of chunks (1: the partials are added without groups)
   int R, restart, nchunk, chunk;  // rows per CTA of the dots and cycle-start kernels
   int nuchunk, uchunk;             // rows per CTA of the update
   int max_iter;
