@@ -48,6 +48,8 @@ constexpr int kPLanesPerRow = 4;                         // lanes per row of the
 constexpr int64_t kPersistWideRow = 128;  // mean entries per row from which a warp takes a row of E
                                           // in global memory (four entries or more per lane)
 
+constexpr int kPersistColumnRows = 128;   // rows per CTA up to which the warps split the columns instead
+
 struct PArgs {
   KPtr P;                  // st, jlast, resid, H, coef, R, restart, N, tol
   PSync* sync;
@@ -64,7 +66,8 @@ struct PArgs {
   int G, rows, max_iter;
   unsigned arrivals;       // arrivals a grid barrier waits for (G; more only in the timeout test)
   int vsm, esm;            // V / E slices in shared memory
-  int wide;                // long rows of E read from global memory: a warp per row
+  int wide;                // long rows of E read from global memory: 1 a warp per row, 2 the columns split
+                           // over the warps (few rows per CTA, one right-hand side)
   int64_t emax, cmax;      // largest E and column-map slice of a CTA (entries)
   int bnorm_given;         // P.bnorm holds |b| (else the first residual norm is |b|)
   int y_zero;              // Y starts at zero: each CTA clears its rows and the first residual is B
@@ -361,9 +364,96 @@ struct ESlice {
   const int32_t* cm;
   const RowInfo* ri;
   int64_t ebase, cbase;  // subtracted from the descriptors' offsets
+  cplx<TV>* pw;          // [rows][kPWarps] sums of the warps' columns (shared, PArgs::wide == 2)
   cplx<TV>* xg;          // [R][cstride] gathered vector at the column-map slice (shared) or null
   int clen, cstride;
 };
+
+// Sums over the warp of four values, the first result in lanes 0-7, the second in 8-15 and so on.
+template <typename TV>
+__device__ __forceinline__ TV p_sum4(TV a, TV b, TV c, TV d, int lane) {
+  const bool h = lane & 16, l = lane & 8;
+  const TV k0 = (h ? c : a) + __shfl_xor_sync(0xffffffffu, h ? a : c, 16);
+  const TV k1 = (h ? d : b) + __shfl_xor_sync(0xffffffffu, h ? b : d, 16);
+  TV k = (l ? k1 : k0) + __shfl_xor_sync(0xffffffffu, l ? k0 : k1, 8);
+  k += __shfl_xor_sync(0xffffffffu, k, 4);
+  k += __shfl_xor_sync(0xffffffffu, k, 2);
+  return k + __shfl_xor_sync(0xffffffffu, k, 1);
+}
+
+// The product for few long rows per CTA and one right-hand side: the warps split the columns (32 at a
+// time, in turn), and a lane takes a column of up to eight rows of one wire, which share their column map:
+// one entry of the map and one gathered value serve them all, and up to 24 loads of E are in flight per
+// lane (three columns; one in float64, for want of registers).  Each warp's sums go to S.pw and are added in warp order.  Entire coupling of 1,000 wires
+// (210 MB of E per product), the whole solve of 8 steps: 0.98 ms with a warp per row, 0.77 ms so.
+template <typename TV, typename TE>
+__device__ void p_product_columns(int mode, const PArgs& a, const ESlice<TV, TE>& S, const cplx<TV>* __restrict__ src,
+                                  cplx<TV>* ys, cplx<TV>* ws, int cnt, int64_t n0, bool on,
+                                  const cplx<TV>* __restrict__ B, cplx<TV>* __restrict__ W, TV& nrm) {
+  constexpr int RT = 8;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  if (on) {
+    for (int t0 = 0, len; t0 < cnt; t0 += len) {
+      const RowInfo ri = S.ri[t0];
+      const RowInfo rl = S.ri[min(t0 + lane, cnt - 1)];  // a wire without columns has its successor's map
+      const unsigned same =
+          __ballot_sync(0xffffffffu, lane < RT && t0 + lane < cnt && rl.cmb == ri.cmb && rl.K == ri.K);
+      len = max(1, __ffs(~same) - 1);
+      const int K = ri.K;
+      const TE* e = S.e + ri.vb;
+      const int32_t* cm = S.cm + ri.cmb;
+      cplx<TV> acc[RT];
+#pragma unroll
+      for (int r = 0; r < RT; ++r) acc[r] = mkc<TV>(0, 0);
+      constexpr int ST = kPT;                      // columns of a pass of all warps
+      constexpr int CB = sizeof(TV) == 4 ? 3 : 1;  // columns of a lane in flight
+      int c = wp * 32 + lane;
+      int32_t q[CB];
+#pragma unroll
+      for (int u = 0; u < CB; ++u) q[u] = c + u * ST < K ? cm[c + u * ST] : 0;
+#pragma unroll 1
+      for (; c < K; c += CB * ST) {
+        cplx<TV> ev[CB][RT], x[CB];
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+#pragma unroll
+          for (int u = 0; u < CB; ++u)
+            if (r < len) ev[u][r] = c + u * ST < K ? ELoad<TV, TE>::ld(e + (int64_t)r * K + c + u * ST) : mkc<TV>(0, 0);
+#pragma unroll
+        for (int u = 0; u < CB; ++u) x[u] = ldcg_c<TV>(src + q[u]);
+#pragma unroll
+        for (int u = 0; u < CB; ++u) q[u] = c + (CB + u) * ST < K ? cm[c + (CB + u) * ST] : 0;
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+#pragma unroll
+          for (int u = 0; u < CB; ++u)
+            if (r < len && c + u * ST < K) cfma(acc[r], ev[u][r], x[u]);
+      }
+#pragma unroll
+      for (int r = 0; r < RT; r += 2)
+        if (r < len) {
+          const TV s = p_sum4<TV>(acc[r].re, acc[r].im, acc[r + 1].re, acc[r + 1].im, lane);
+          const int rr = r + (lane >> 4);
+          if ((lane & 7) == 0 && rr < len)
+            reinterpret_cast<TV*>(S.pw + (t0 + rr) * kPWarps + wp)[(lane >> 3) & 1] = s;
+        }
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; on && t < cnt; t += kPT) {
+    cplx<TV> s = mkc<TV>(0, 0);
+    for (int w = 0; w < kPWarps; ++w) s = s + S.pw[t * kPWarps + w];
+    const int64_t n = n0 + t;
+    if (mode == 0) {
+      ws[t] = ys[t] + s;
+    } else {
+      const cplx<TV> r = B[n] - (src[n] + s);
+      ys[t] = r;
+      W[n] = r;
+      nrm = fma(r.re, r.re, fma(r.im, r.im, nrm));
+    }
+  }
+}
 
 // Rows of the CTA times A = I + E for the R right-hand sides of `src`.
 // mode 0 (Arnoldi): ws = u + E u for the pending vector u (own rows in ys, all rows in src).
@@ -405,6 +495,13 @@ __device__ void p_product(int mode, const PArgs& a, const ESlice<TV, TE>& S, con
           if (col[u] >= 0 && on[b]) S.xg[b * S.cstride + q0 + u * kPT] = v[u][b];
     }
     __syncthreads();
+  }
+  if constexpr (RB == 1) {
+    if (a.wide == 2) {
+      p_product_columns<TV, TE>(mode, a, S, src, ys, ws, cnt, n0, on[0], B, W, nrm[0]);
+      if (mode == 1) p_norm_partials<TV, RB>(nrm, R, a.G, (TV*)a.partn, red);
+      return;
+    }
   }
   if (!S.xg && a.wide) {
     // Long rows streamed from global memory (entire coupling: 5,128 entries a row at 1,000 wires,
@@ -605,6 +702,7 @@ __global__ void __launch_bounds__(kPT, 1) k_gmres_persist(PArgs a) {
   S.ri = a.rinfo + n0;
   S.ebase = 0;
   S.cbase = 0;
+  S.pw = reinterpret_cast<C*>(sm_raw + L.total);
   S.xg = nullptr;
   S.clen = 0;
   S.cstride = 0;
@@ -975,7 +1073,10 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   }
   const int esm = emax >= mean_e && emax > 0 ? 1 : 0;
   if (!esm) emax = cmax = 0;
-  const size_t smem = persist_layout(RB, R, restart, prows, hown, cb, eb, vsm, esm, emax, cmax).total;
+  size_t smem = persist_layout(RB, R, restart, prows, hown, cb, eb, vsm, esm, emax, cmax).total;
+  const size_t pw = cb * kPWarps * (size_t)prows;
+  const bool columns = wide && !esm && R == 1 && prows <= kPersistColumnRows && smem + pw <= limit;
+  if (columns) smem += pw;
   if (smem > limit) return SWM_OK;
   int occ = 0;
   SWM_CK(occupancy_cached(fn, kPT, smem, &occ));
@@ -999,7 +1100,7 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   pa.max_iter = max_iter;
   pa.vsm = vsm;
   pa.esm = esm;
-  pa.wide = wide && !esm ? 1 : 0;
+  pa.wide = columns ? 2 : wide && !esm ? 1 : 0;
   pa.emax = emax;
   pa.cmax = cmax;
   pa.bnorm_given = Bf.bnorm_given;
