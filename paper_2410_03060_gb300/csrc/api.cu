@@ -443,6 +443,7 @@ int swm_set_cloud(swm_ctx* ctx, int64_t nw, const double* centres, const double*
   ctx->pattern_ok = false;
   ctx->rowwire = nullptr;
   ctx->wrec = ctx->pkrec = ctx->pack = nullptr;
+  ctx->worder = nullptr;
   ctx->pack_refused = false;
   ctx->nw = nw;
   auto& G = ctx->cloud_bufs;
@@ -539,6 +540,7 @@ int swm_build(swm_ctx* ctx, double k, double r_c, int precision) {
     ctx->pattern_ok = false;
     ctx->rowwire = nullptr;
     ctx->wrec = ctx->pkrec = nullptr;
+    ctx->worder = nullptr;
     ctx->uoff = nullptr;
     ctx->uoff_user = nullptr;
     SWM_TRY(build_pattern(ctx));

@@ -122,6 +122,7 @@ struct swm_ctx {
   int32_t* rowwire = nullptr;  // [N] internal wire of each scalar row
   void* wrec = nullptr;        // [nw] wire records of product form 75 in its order (built by the
                                // first solve that may use it after a pattern build)
+  int32_t* worder = nullptr;   // [nw] wires by (rows, columns) within windows, with the pattern
   void* pkrec = nullptr;       // [nw] wire records of product form 76 (product_pack.cu), with the pattern
   void* pack = nullptr;        // E and the column map in that order, one record per wire, with the values
   bool pack_refused = false;   // no memory was left for it (until the next cloud)
@@ -314,6 +315,8 @@ int build_wire_order(swm_ctx* ctx);
 // after a build; krylov_common.cuh declares the product's launch).  *ok = 0: E is too large for a second
 // copy, or no memory was left for it.
 int ensure_pack(swm_ctx* ctx, bool* ok);
+// product_pack.cu: the wire order of the float64 products (worder; once per pattern)
+int ensure_row_order(swm_ctx* ctx);
 // row descriptors of E (built once per build) and x = M^-1 y into ctx->Xv
 int ensure_rowinfo(swm_ctx* ctx);
 // y = y0 (ctx->guess, complex128) or 0 at the start of a solve, in the vector precision

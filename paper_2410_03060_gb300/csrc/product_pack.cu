@@ -49,9 +49,11 @@ __device__ __forceinline__ int pack_mp(int m) { return (m + 1) & ~1; }
 __device__ __forceinline__ int pack_k(int K) { return (K + 1) & ~1; }
 __device__ __forceinline__ int pack_cb(int K) { return (4 * K + 15) & ~15; }
 
-// One CTA per window: bitonic sort of (rows, columns, position); then the record sizes in order.
+// One CTA per window: bitonic sort of (rows, columns, position); then the record sizes in order, or, with
+// `order`, only the wires' numbers.
 __global__ void __launch_bounds__(1024) k_pack_order(int64_t nw, Layout lay, const int64_t* __restrict__ off,
-                                                     PackRec* __restrict__ rec, int64_t* __restrict__ bytes) {
+                                                     PackRec* __restrict__ rec, int64_t* __restrict__ bytes,
+                                                     int32_t* __restrict__ order) {
   __shared__ unsigned long long key[kPackWin];
   const int64_t base = (int64_t)blockIdx.x * kPackWin;
   for (int t = threadIdx.x; t < kPackWin; t += blockDim.x) {
@@ -79,6 +81,10 @@ __global__ void __launch_bounds__(1024) k_pack_order(int64_t nw, Layout lay, con
     const int64_t i = base + t;
     if (i >= nw) continue;
     const int64_t p = base + (int64_t)(key[t] & 0xffffffffu);
+    if (order) {
+      order[i] = (int32_t)p;
+      continue;
+    }
     PackRec r;
     r.at = 0;
     r.row0 = (int32_t)off[p];
@@ -349,7 +355,7 @@ static int make_pack(swm_ctx* ctx) {
     if (rc >= 0) rc = dalloc(ctx, tmp, (void**)&at, sizeof(int64_t) * (nw + 1));
     if (rc >= 0) {
       PackRec* rec = reinterpret_cast<PackRec*>(recs);
-      k_pack_order<<<(unsigned)ceil_div(nw, kPackWin), 1024, 0, ctx->stream>>>(nw, ctx->offd, ctx->off, rec, bytes);
+      k_pack_order<<<(unsigned)ceil_div(nw, kPackWin), 1024, 0, ctx->stream>>>(nw, ctx->offd, ctx->off, rec, bytes, nullptr);
       SWM_LAUNCHED();
       const void* in[1] = {bytes};
       const int is64[1] = {1};
@@ -382,6 +388,21 @@ int ensure_pack(swm_ctx* ctx, bool* ok) {
   release_spare(ctx);
   ctx->pack_refused = true;
   *ok = false;
+  return SWM_OK;
+}
+
+int ensure_row_order(swm_ctx* ctx) {
+  if (ctx->worder || ctx->nw <= 0 || ctx->nw > INT32_MAX) return SWM_OK;
+  // under a caller's capture the order would not exist before the graph runs: the wires as they lie
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  SWM_CK(cudaStreamIsCapturing(ctx->stream, &cs));
+  if (cs != cudaStreamCaptureStatusNone) return SWM_OK;
+  int32_t* w = nullptr;
+  SWM_TRY(dalloc(ctx, ctx->pattern_bufs, (void**)&w, sizeof(int32_t) * ctx->nw));
+  k_pack_order<<<(unsigned)ceil_div(ctx->nw, kPackWin), 1024, 0, ctx->stream>>>(ctx->nw, ctx->offd, ctx->off, nullptr,
+                                                                               nullptr, w);
+  SWM_LAUNCHED();
+  ctx->worder = w;
   return SWM_OK;
 }
 
