@@ -159,6 +159,79 @@ __global__ void __launch_bounds__(kRows) k_spmv(KPtr P, const RowInfo* __restric
   }
 }
 
+// The same for one right-hand side, eight lanes per wire: the rows of a wire share their column map, so a
+// lane's column and gathered value serve up to eight rows.  Bound by latency (offsets, column, then E and
+// the gather; rows are 40 entries long): with 80 registers, three CTAs of eight warps, DRAM ran at 45 % and
+// nothing was gained on a row per eight lanes.  CTAs of four warps at 64 registers (eight per SM, a few
+// spills) keep more of the short warps in flight; one column at a time in 48 registers was 2 % slower.
+// 400,001 wires, one incidence: the call 18.26 -> 17.25 ms.
+constexpr int kOneThreads = 128;
+template <typename TV, typename TE, bool RES>
+__global__ void __launch_bounds__(kOneThreads, sizeof(TV) == 4 ? 8 : 4)
+    k_spmv_one(KPtr P, const int64_t* __restrict__ off, Layout lay, int64_t nw, const TE* __restrict__ E,
+               const cplx<TV>* __restrict__ U, cplx<TV>* __restrict__ Wv, const cplx<TV>* __restrict__ B) {
+  if (!RES && (P.st->cycle_done || P.st->j >= P.st->jmax || !P.active[0])) return;
+  const int64_t p = (blockIdx.x * (int64_t)kOneThreads + threadIdx.x) / kG;
+  const int sub = threadIdx.x % kG;
+  int m = 0, K = 0;
+  int64_t n0 = 0;
+  const TE* Ep = E;
+  const int32_t* cm = lay.colmap;
+  if (p < nw) {
+    n0 = off[p];
+    m = (int)(off[p + 1] - n0);
+    K = lay.K[p];
+    Ep = E + lay.rowbase[p];
+    cm += lay.cmbase[p];
+  }
+  const int mw = __reduce_max_sync(0xffffffffu, m);
+  for (int i0 = 0; i0 < mw; i0 += 8) {
+    const int mm = min(8, m - i0);
+    const TE* e = Ep + (int64_t)i0 * K + sub;
+    cplx<TV> acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = mkc<TV>(0, 0);
+    int c = sub;
+    int32_t q0 = c < K ? cm[c] : 0, q1 = c + kG < K ? cm[c + kG] : 0;
+    for (; c < K; c += 2 * kG, e += 2 * kG) {
+      const bool two = c + kG < K;
+      cplx<TV> e0[8], e1[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < mm) {
+          e0[i] = ELoad<TV, TE>::ld(e + (int64_t)i * K);
+          e1[i] = two ? ELoad<TV, TE>::ld(e + (int64_t)i * K + kG) : mkc<TV>(0, 0);
+        }
+      const cplx<TV> x0 = U[q0], x1 = U[q1];
+      q0 = c + 2 * kG < K ? cm[c + 2 * kG] : 0;
+      q1 = c + 3 * kG < K ? cm[c + 3 * kG] : 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < mm) {
+          cfma(acc[i], e0[i], x0);
+          if (two) cfma(acc[i], e1[i], x1);
+        }
+    }
+    __syncwarp();
+    // sums over the eight lanes, lane i left with row i
+    const bool h = sub & 4, l = sub & 2, z = sub & 1;
+    auto xch = [&](cplx<TV> keep, cplx<TV> give, int o) {
+      keep.re += __shfl_xor_sync(0xffffffffu, give.re, o);
+      keep.im += __shfl_xor_sync(0xffffffffu, give.im, o);
+      return keep;
+    };
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = xch(h ? acc[i + 4] : acc[i], h ? acc[i] : acc[i + 4], 4);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) acc[i] = xch(l ? acc[i + 2] : acc[i], l ? acc[i] : acc[i + 2], 2);
+    const cplx<TV> s = xch(z ? acc[1] : acc[0], z ? acc[0] : acc[1], 1);
+    if (sub < mm) {
+      const int64_t n = n0 + i0 + sub;
+      Wv[n] = RES ? B[n] - (U[n] + s) : U[n] + s;
+    }
+  }
+}
+
 // Product with many right-hand sides, part 0: the pending vectors U (right-hand-side major,
 // [R][N]) copied to right-hand-side minor order Xt[N][R] through shared-memory tiles of 32 rows x
 // 32 right-hand sides, so that the product below reads the values of all right-hand sides at a
@@ -1727,7 +1800,10 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
     cplx<TV>* dst = RS ? U : Wv;
     const dim3 gsp((unsigned)ceil_div(N * kG, kRows), (unsigned)ceil_div(R, std::min(b, 16)));
     switch (b) {
-      case 1: k_spmv<TV, TE, 1, RS><<<gsp, kRows, 0, s>>>(P, ri, ctx->offd.colmap, E, src, dst, Bv); break;
+      case 1:
+        k_spmv_one<TV, TE, RS><<<(unsigned)ceil_div(ctx->nw * kG, kOneThreads), kOneThreads, 0, s>>>(
+            P, ctx->off, ctx->offd, ctx->nw, E, src, dst, Bv);
+        break;
       case 4: k_spmv<TV, TE, 4, RS><<<gsp, kRows, 0, s>>>(P, ri, ctx->offd.colmap, E, src, dst, Bv); break;
       case 16: k_spmv<TV, TE, 16, RS><<<gsp, kRows, 0, s>>>(P, ri, ctx->offd.colmap, E, src, dst, Bv); break;
       case kMinor: {

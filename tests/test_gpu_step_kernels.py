@@ -1,4 +1,4 @@
-"""GPU test of the per-kernel GMRES steps (dots with partial sums in groups of chunks, the wire-tiled float64
+"""GPU test of the per-kernel GMRES steps (the product of one incidence by wires, dots with partial sums in groups of chunks, the wire-tiled float64
 product over the sorted wires) against the persistent solve: row counts that leave the last chunk, piece and
 group short, one incidence (more than 64 chunks) and several, from zero and with a restart."""
 import numpy as np
@@ -27,9 +27,10 @@ def _solve(cl, prec, inc, tol, restart, persist, monkeypatch):
 
 
 @pytest.mark.parametrize("prec,tol,bound", [(1, 1e-5, 2e-4), (0, 1e-10, 1e-8)])
-@pytest.mark.parametrize("nw,n_inc,restart", [(3301, 1, 50), (4203, 9, 4), (257, 40, 50)])
-def test_step_kernels_match_the_persistent_solve(nw, n_inc, restart, prec, tol, bound, monkeypatch):
-    cl = cloud_uniform_cube(nw, 2.2 * nw ** (1 / 3), seed=nw)
+@pytest.mark.parametrize("nw,n_inc,restart,nseg", [(3301, 1, 50, None), (61, 1, 50, 16), (33, 1, 50, 2),
+                                                   (4203, 9, 4, None), (257, 40, 50, None)])
+def test_step_kernels_match_the_persistent_solve(nw, n_inc, restart, nseg, prec, tol, bound, monkeypatch):
+    cl = cloud_uniform_cube(nw, 2.2 * nw ** (1 / 3), seed=nw, nseg=nseg)
     rng = np.random.default_rng(n_inc)
     inc = np.stack([rng.uniform(0, 3, n_inc), rng.uniform(0, 6, n_inc), rng.uniform(0, 1, n_inc)], 1)
     a = _solve(cl, prec, inc, tol, restart, False, monkeypatch)
