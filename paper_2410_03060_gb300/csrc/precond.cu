@@ -230,12 +230,14 @@ __global__ void __launch_bounds__(kFormThreads) k_form_E(int64_t nb, const int32
   }
 }
 
-// The same, one warp per block and a lane per entry: the float64 form.  There the multiply-adds issue
-// sixteen times slower than the loads they wait for, and a lane per column spends more of them on lanes
-// past the row and column counts of its own block (10,007 wires: 118 us here, 182 us by columns).
+// The same, one warp per block and a lane per entry: the form of float64, whose multiply-adds issue sixteen
+// times slower than the loads they wait for (a lane per column spends more of them on lanes past the row
+// and column counts of its own block: 10,007 wires 118 us here, 182 us by columns), and of small clouds,
+// whose few warps by columns each have a longer chain (7,856 blocks 8.9 us here, 12.2 us by columns).
+template <typename TV>
 __global__ void k_form_E_entries(int64_t nb, const int32_t* __restrict__ col, const int64_t* __restrict__ bt,
-                         const int32_t* __restrict__ m, Layout full, Layout offd, const c128* __restrict__ Z,
-                         const int64_t* __restrict__ moff, const c128* __restrict__ Minv, c128* __restrict__ E) {
+                         const int32_t* __restrict__ m, Layout full, Layout offd, const cplx<TV>* __restrict__ Z,
+                         const int64_t* __restrict__ moff, const cplx<TV>* __restrict__ Minv, cplx<TV>* __restrict__ E) {
   const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (b >= nb) return;
@@ -246,10 +248,10 @@ __global__ void k_form_E_entries(int64_t nb, const int32_t* __restrict__ col, co
   const int Kf = full.K[p], Ko = offd.K[p];
   const int64_t zb = full.rowbase[p] + full.colpos[b];
   const int64_t eb = offd.rowbase[p] + offd.colpos[b];
-  const c128* Mi = Minv + moff[q];
+  const cplx<TV>* Mi = Minv + moff[q];
   for (int e = lane; e < mp * mq; e += 32) {
     const int i = e / mq, j = e % mq;
-    c128 acc = mkc(0.0, 0.0);
+    cplx<TV> acc = mkc<TV>(0, 0);
     for (int l = 0; l < mq; ++l) cfma(acc, Z[zb + (int64_t)i * Kf + l], Mi[l * mq + j]);
     E[eb + (int64_t)i * Ko + j] = acc;
   }
@@ -286,19 +288,24 @@ int precond_invert(swm_ctx* ctx, cudaStream_t s) {
 // E = Z M^-1 off the diagonal, on the context's stream (after the fill and the inversion).
 int precond_form_E(swm_ctx* ctx) {
   const unsigned g1 = (unsigned)std::max<int64_t>(1, ceil_div(ctx->nb * 32, 256));
-  // 32 blocks per warp, fewer (down to 4, one pass over their columns) while that leaves warps to spare
-  int per = 32;
-  while (per > 4 && ctx->nb < (int64_t)per * 16 * std::max(ctx->nsm, 1)) per >>= 1;
+  // By columns from about 256 blocks per SM (8 warps of 32); 16 blocks per warp while that is few warps.
+  const int64_t nsm = std::max(ctx->nsm, 1);
+  const bool columns = ctx->prec != SWM_C128 && ctx->nb >= 256 * nsm;
+  const int per = ctx->nb >= 512 * nsm ? 32 : 16;
   const unsigned g2 = (unsigned)std::max<int64_t>(1, ceil_div(ctx->nb, (int64_t)per * (kFormThreads / 32)));
   ctx->prof_begin(SWM_K_FORM_E);
   if (ctx->prec == SWM_C128)
-    k_form_E_entries<<<g1, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
-                                                  (const c128*)ctx->Z, ctx->minv_off, (const c128*)ctx->Minv,
-                                                  (c128*)ctx->Zp);
-  else
+    k_form_E_entries<double><<<g1, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
+                                                          (const c128*)ctx->Z, ctx->minv_off, (const c128*)ctx->Minv,
+                                                          (c128*)ctx->Zp);
+  else if (columns)
     k_form_E<<<g2, kFormThreads, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
-                                                 (const c64*)ctx->Z, ctx->minv_off, (const c64*)ctx->Minv,
-                                                 (c64*)ctx->Zp, per);
+                                                   (const c64*)ctx->Z, ctx->minv_off, (const c64*)ctx->Minv,
+                                                   (c64*)ctx->Zp, per);
+  else
+    k_form_E_entries<float><<<g1, 256, 0, ctx->stream>>>(ctx->nb, ctx->col, ctx->bt, ctx->m, ctx->full, ctx->offd,
+                                                         (const c64*)ctx->Z, ctx->minv_off, (const c64*)ctx->Minv,
+                                                         (c64*)ctx->Zp);
   ctx->prof_end(SWM_K_FORM_E);
   SWM_LAUNCHED();
   return SWM_OK;
