@@ -383,8 +383,8 @@ __device__ __forceinline__ TV p_sum4(TV a, TV b, TV c, TV d, int lane) {
 
 // The product for few long rows per CTA and one right-hand side: the warps split the columns (32 at a
 // time, in turn), and a lane takes a column of up to eight rows of one wire, which share their column map:
-// one entry of the map and one gathered value serve them all, and up to 24 loads of E are in flight per
-// lane (three columns; one in float64, for want of registers).  Each warp's sums go to S.pw and are added in warp order.  Entire coupling of 1,000 wires
+// one entry of the map and one gathered value serve them all, and up to 16 loads of E are in flight per
+// lane (two columns; one in float64; more spill registers, also in the other paths of the kernel).  Each warp's sums go to S.pw and are added in warp order.  Entire coupling of 1,000 wires
 // (210 MB of E per product), the whole solve of 8 steps: 0.98 ms with a warp per row, 0.77 ms so.
 template <typename TV, typename TE>
 __device__ void p_product_columns(int mode, const PArgs& a, const ESlice<TV, TE>& S, const cplx<TV>* __restrict__ src,
@@ -406,7 +406,7 @@ __device__ void p_product_columns(int mode, const PArgs& a, const ESlice<TV, TE>
 #pragma unroll
       for (int r = 0; r < RT; ++r) acc[r] = mkc<TV>(0, 0);
       constexpr int ST = kPT;                      // columns of a pass of all warps
-      constexpr int CB = sizeof(TV) == 4 ? 3 : 1;  // columns of a lane in flight
+      constexpr int CB = sizeof(TV) == 4 ? 2 : 1;  // columns of a lane in flight
       int c = wp * 32 + lane;
       int32_t q[CB];
 #pragma unroll
