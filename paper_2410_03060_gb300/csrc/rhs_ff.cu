@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kFFThreads) k_far_partial(Geo geo, int64_t nw,
     if (!on) continue;
     for (int t = 0; t < cnt; ++t) {
       const Wire& w = sw[t];
+      if (w.n < 2) continue;  // a wire without unknowns (the stateless entries take the counts unchecked)
       const double beta = k * (rh[0] * w.t[0] + rh[1] * w.t[1] + rh[2] * w.t[2]);
       const double x = rh[0] * w.c[0] + rh[1] * w.c[1] + rh[2] * w.c[2];
       double sa, ca, sc, cz;
