@@ -39,6 +39,20 @@ constexpr int kMinorR = 12;  // right-hand sides from which the large-system pro
 constexpr int kG = 8;       // lanes per scalar row in the block-sparse product
 constexpr int kMaxChunk = 2048;  // rows per CTA of the Gram-Schmidt kernels, at most
 
+// A solve's workspace stays in the context only when all of its buffers exist: an allocation that fails
+// (or any other way out before `complete`) gives back what was there and forgets the workspace, so the
+// next solve starts over instead of running on null buffers.
+struct WorkspaceGuard {
+  swm_ctx* ctx;
+  bool complete = false;
+  ~WorkspaceGuard() {
+    if (complete) return;
+    dfree_group(ctx, ctx->kry_bufs);
+    std::free(ctx->kry_ws);
+    ctx->kry_ws = nullptr;
+  }
+};
+
 template <typename T>
 __device__ __forceinline__ bool finite_c(cplx<T> z) {
   return isfinite((double)z.re) && isfinite((double)z.im);
@@ -1706,6 +1720,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
     if (!ws) return ctx->fail(SWM_ENOMEM, "host allocation failed");
     ctx->kry_ws = ws;
     ctx->kry_ws_bytes = sizeof(Workspace);
+    WorkspaceGuard guard{ctx};
     std::memcpy(ws->key, key, sizeof(key));
     auto& K = ctx->kry_bufs;
     SWM_TRY(dalloc(ctx, K, (void**)&P.st, sizeof(KState)));
@@ -1742,6 +1757,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
       SWM_TRY(dalloc(ctx, K, (void**)&ws->ppn, sizeof(double) * (size_t)R * ctx->nsm));
     }
     ws->P = P;
+    guard.complete = true;
   } else {
     const double tol_now = P.tol;
     const int max_iter_now = P.max_iter;
@@ -2433,6 +2449,7 @@ int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
     if (!ws) return ctx->fail(SWM_ENOMEM, "host allocation failed");
     ctx->kry_ws = ws;
     ctx->kry_ws_bytes = sizeof(Workspace);
+    WorkspaceGuard guard{ctx};
     std::memcpy(ws->key, key, sizeof(key));
     auto& K = ctx->kry_bufs;
     BPtr B{};
@@ -2458,6 +2475,7 @@ int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
     for (auto v : vecs) SWM_TRY(dalloc(ctx, K, (void**)v, sizeof(cplx<TV>) * R * N));
     if (xt) SWM_TRY(dalloc(ctx, K, (void**)&ws->Xt, sizeof(cplx<TV>) * (size_t)xst * N));
     ws->B = B;
+    guard.complete = true;
   }
   BPtr B = ws->B;
   B.tol = tol;
@@ -3016,6 +3034,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
     if (!ws) return ctx->fail(SWM_ENOMEM, "host allocation failed");
     ctx->kry_ws = ws;
     ctx->kry_ws_bytes = sizeof(Workspace);
+    WorkspaceGuard guard{ctx};
     std::memcpy(ws->key, key, sizeof(key));
     auto& K = ctx->kry_bufs;
     BmPtr B{};
@@ -3047,6 +3066,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       SWM_CK(cudaMemsetAsync(*v, 0, vbytes, st));
     }
     ws->B = B;
+    guard.complete = true;
   }
   BmPtr B = ws->B;
   B.tol = tol;
