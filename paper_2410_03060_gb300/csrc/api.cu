@@ -445,7 +445,7 @@ int swm_set_cloud(swm_ctx* ctx, int64_t nw, const double* centres, const double*
   ctx->wrec = ctx->pkrec = ctx->pack = nullptr;
   ctx->worder = nullptr;
   ctx->pack_refused = false;
-  ctx->nw = nw;
+  ctx->nw = 0;  // no cloud until every array exists and has been checked
   auto& G = ctx->cloud_bufs;
   SWM_TRY(dalloc(ctx, G, (void**)&ctx->u_c, sizeof(double) * 3 * nw));
   SWM_TRY(dalloc(ctx, G, (void**)&ctx->u_t, sizeof(double) * 3 * nw));
@@ -494,9 +494,9 @@ int swm_set_cloud(swm_ctx* ctx, int64_t nw, const double* centres, const double*
     if (hf[0] & 8) m += " radius <= 0;";
     if (hf[0] & 16) m += " segment count outside [2, " + std::to_string(kMaxSeg) + "];";
     dfree_group(ctx, ctx->cloud_bufs);
-    ctx->nw = 0;
     return ctx->fail(SWM_EINVAL, m);
   }
+  ctx->nw = nw;
   ctx->max_ns = hf[1];
   ctx->stats = swm_stats{};
   ctx->stats.nw = nw;
