@@ -315,6 +315,8 @@ int build_wire_order(swm_ctx* ctx);
 // after a build; krylov_common.cuh declares the product's launch).  *ok = 0: E is too large for a second
 // copy, or no memory was left for it.
 int ensure_pack(swm_ctx* ctx, bool* ok);
+// product_pack.cu: what a build's copy costs, in ms
+double pack_ms(const swm_ctx* ctx);
 // product_pack.cu: the wire order of the float64 products (worder; once per pattern)
 int ensure_row_order(swm_ctx* ctx);
 // row descriptors of E (built once per build) and x = M^-1 y into ctx->Xv

@@ -3013,8 +3013,15 @@ __global__ void __launch_bounds__(256) k_minor_to_major(int64_t N, int R, int xs
     for (int t = lane; t < cnt; t += 32) Y[(int64_t)r * N + n0 + t] = tile[t * ts + r];
 }
 
+// The timed choice weighs a form's product, as often as a solve of ten to twenty steps runs it, against
+// what every build pays for the form: the sort of form 75's order (40 to 51 us from 300 to 300,000 wires)
+// or the copy of form 76 (pack_ms).  On small clouds these decide: 1,000 wires x 4, 26 products of 8.3 us
+// in form 74, 9.7 in 75, 8.7 in 76: the call took 2.48 ms with 74, 2.57 with 76 chosen by the product alone.
+constexpr int kTuneProducts = 32;
+constexpr double kOrderMs = 0.045;
+constexpr float kTuneAllMs = 0.1f;  // products up to which every form is timed
+
 int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
-  SWM_TRY(build_wire_order(ctx));  // the order of product form 75, once per pattern
   cudaStream_t st = ctx->stream;
   const int R = ctx->n_rhs;
   const int64_t N = ctx->N;
@@ -3130,16 +3137,19 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       form = found;
     } else {
       bool packed = false;
+      SWM_TRY(build_wire_order(ctx));
       SWM_TRY(ensure_pack(ctx, &packed));
-      // each shape once untimed and once timed on b (the product is idempotent)
+      // Each shape once untimed and once timed on b (the product is idempotent), the sorted forms first.
+      // Form 76 leads from 30,000 wires (by up to 4 on clusters), 74, 75 and 69 on smaller clouds; the others
+      // are timed while a product is short, where one of them can be the best and their timing costs little.
       cudaEvent_t e0, e1;
       SWM_CK(cudaEventCreate(&e0));
       SWM_CK(cudaEventCreate(&e1));
-      float best = 0.f;
-      // With its copy of E form 76 is the fastest at 50,000 clustered wires and up (by 1.15 to 4) and within 2 %
-      // of the fastest on sparse and small clouds, where 73 or 75 lead; the others led nowhere by more than 1 %.
-      for (int f : {68, 69, 70, 71, 72, 73, 74, 75, 76}) {
-        if (packed ? f != 73 && f < 75 : f == 76) continue;
+      double best = 0.0;
+      float shortest = 0.f;
+      for (int f : {76, 75, 73, 74, 69, 68, 70, 71, 72}) {
+        if (!packed && f == 76) continue;
+        if (packed && f != 73 && f < 75 && shortest > kTuneAllMs) break;
         form = f;
         SWM_TRY(product(st, Bt, Vv, std::true_type{}));
         SWM_CK(cudaEventRecord(e0, st));
@@ -3148,8 +3158,10 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
         SWM_CK(cudaEventSynchronize(e1));
         float ms = 0.f;
         SWM_CK(cudaEventElapsedTime(&ms, e0, e1));
-        if (best == 0.f || ms < best) {
-          best = ms;
+        if (shortest == 0.f || ms < shortest) shortest = ms;
+        const double cost = kTuneProducts * ms + (f == 76 ? pack_ms(ctx) : f == 75 ? kOrderMs : 0.0);
+        if (best == 0.0 || cost < best) {
+          best = cost;
           found = f;
         }
       }
@@ -3167,6 +3179,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
     SWM_TRY(ensure_pack(ctx, &packed));
     if (!packed) form = 75;
   }
+  if (form == 75) SWM_TRY(build_wire_order(ctx));  // once per pattern
   ctx->stats.step_rhs_block = form;
   const unsigned gC = (unsigned)B.nchunk;
   auto launch_steps = [&](cudaStream_t s, int n) -> int {

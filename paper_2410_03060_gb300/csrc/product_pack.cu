@@ -391,6 +391,10 @@ int ensure_pack(swm_ctx* ctx, bool* ok) {
   return SWM_OK;
 }
 
+// Sort (39 to 46 us), scan and placement (about 10 us) and fill (4 us and 0.4 ms per GB: 29 MB 16 us, 298 MB
+// 121 us), measured from 300 to 300,000 wires.
+double pack_ms(const swm_ctx* ctx) { return 0.06 + 0.4e-9 * (double)pack_most(ctx); }
+
 int ensure_row_order(swm_ctx* ctx) {
   if (ctx->worder || ctx->nw <= 0 || ctx->nw > INT32_MAX) return SWM_OK;
   // under a caller's capture the order would not exist before the graph runs: the wires as they lie
