@@ -62,10 +62,8 @@ static void give_back(swm_ctx* ctx, const Buf& b) {
     cudaFreeAsync(b.p, ctx->stream);
 }
 
-bool release_spare(swm_ctx* ctx) {
-  bool any = !ctx->free_list.empty();
-  for (auto& b : ctx->free_list) give_back(ctx, b);
-  ctx->free_list.clear();
+bool drop_pack(swm_ctx* ctx) {
+  bool any = false;
   auto drop = [&](std::vector<Buf>& group, void** p) {
     for (size_t i = 0; *p && i < group.size(); ++i)
       if (group[i].p == *p) {
@@ -78,6 +76,13 @@ bool release_spare(swm_ctx* ctx) {
   drop(ctx->build_bufs, &ctx->pack);
   drop(ctx->pattern_bufs, &ctx->pkrec);
   return any;
+}
+
+bool release_spare(swm_ctx* ctx) {
+  const bool any = !ctx->free_list.empty();
+  for (auto& b : ctx->free_list) give_back(ctx, b);
+  ctx->free_list.clear();
+  return drop_pack(ctx) || any;
 }
 
 int dalloc(swm_ctx* ctx, std::vector<Buf>& group, void** out, size_t bytes) {

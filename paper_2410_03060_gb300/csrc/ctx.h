@@ -241,6 +241,8 @@ int dalloc(swm_ctx* ctx, std::vector<Buf>& group, void** out, size_t bytes);
 // and product form 76's copy of E (a solve that wants it makes it again).  False if there was nothing.
 // dalloc does so before it reports that an allocation failed.
 bool release_spare(swm_ctx* ctx);
+// Gives back form 76's copy of E alone.  False if there was none.
+bool drop_pack(swm_ctx* ctx);
 void dfree_group(swm_ctx* ctx, std::vector<Buf>& group);
 
 #define SWM_CK(call)                                                                 \

@@ -3137,6 +3137,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       form = found;
     } else {
       bool packed = false;
+      const bool had_pack = ctx->pack != nullptr;
       SWM_TRY(build_wire_order(ctx));
       SWM_TRY(ensure_pack(ctx, &packed));
       // Each shape once untimed and once timed on b (the product is idempotent), the sorted forms first.
@@ -3172,6 +3173,7 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
       std::memcpy(t.shape, shape, sizeof(shape));
       t.rb = form;
       ctx->tuned.push_back(t);
+      if (form != 76 && !had_pack) drop_pack(ctx);  // made for the timing alone
     }
   }
   if (form == 76) {  // without its copy of E: form 75, the same sums from E itself

@@ -348,23 +348,23 @@ static int make_pack(swm_ctx* ctx) {
   SWM_CK(allow_max_dyn_smem((const void*)k_spmv_pack<false>, ctx->smem_optin));
   if (!ctx->pkrec) {
     std::vector<Buf> tmp;
-    void* recs = nullptr;
     int64_t *bytes = nullptr, *at = nullptr;
-    int rc = dalloc(ctx, ctx->pattern_bufs, &recs, sizeof(PackRec) * nw);
+    int rc = dalloc(ctx, ctx->pattern_bufs, &ctx->pkrec, sizeof(PackRec) * nw);
     if (rc >= 0) rc = dalloc(ctx, tmp, (void**)&bytes, sizeof(int64_t) * nw);
     if (rc >= 0) rc = dalloc(ctx, tmp, (void**)&at, sizeof(int64_t) * (nw + 1));
+    if (rc >= 0 && !ctx->pkrec) rc = SWM_ENOMEM;  // given back to make room
     if (rc >= 0) {
-      PackRec* rec = reinterpret_cast<PackRec*>(recs);
+      PackRec* rec = reinterpret_cast<PackRec*>(ctx->pkrec);
       k_pack_order<<<(unsigned)ceil_div(nw, kPackWin), 1024, 0, ctx->stream>>>(nw, ctx->offd, ctx->off, rec, bytes, nullptr);
       SWM_LAUNCHED();
       const void* in[1] = {bytes};
       const int is64[1] = {1};
       int64_t* out[1] = {at};
       rc = exclusive_scan_multi(ctx, 1, in, is64, out, nw);
+      if (rc >= 0 && !ctx->pkrec) rc = SWM_ENOMEM;
       if (rc >= 0) {
         k_pack_place<<<(unsigned)ceil_div(nw, 256), 256, 0, ctx->stream>>>(nw, at, rec);
         SWM_LAUNCHED();
-        ctx->pkrec = recs;
       }
     }
     dfree_group(ctx, tmp);
@@ -383,11 +383,15 @@ static int make_pack(swm_ctx* ctx) {
 int ensure_pack(swm_ctx* ctx, bool* ok) {
   *ok = pack_most(ctx) <= kPackMost && !ctx->pack_refused;
   if (!*ok) return SWM_OK;
+  const std::string err = ctx->err;
   const int rc = make_pack(ctx);
+  if (rc >= 0) return rc;
+  drop_pack(ctx);  // what there is of it is not complete
+  *ok = false;
   if (rc != SWM_ENOMEM) return rc;
+  ctx->err = err;  // the solve goes on without the copy
   release_spare(ctx);
   ctx->pack_refused = true;
-  *ok = false;
   return SWM_OK;
 }
 
