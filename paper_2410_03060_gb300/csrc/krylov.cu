@@ -28,6 +28,7 @@
 #include "common.cuh"
 #include "ctx.h"
 #include "krylov_common.cuh"
+#include "lane_sums.cuh"
 
 namespace swm {
 
@@ -1270,22 +1271,6 @@ __device__ void dots_tail(const KPtr& P, int j, int r, bool closing, const c128*
   if (threadIdx.x == 0) step_arrive(P, j, closing);
 }
 
-// Sums over the warp of eight values: lanes 4 i .. 4 i + 3 return that of v[i].  Each of the first three
-// exchanges halves the number of values a lane carries (9 additions for 8 sums; one sum after the other
-// takes 40, which in float64 cost half as much as reading the rows).
-template <typename TV>
-__device__ __forceinline__ TV warp_sum8(const TV (&v)[8], int lane) {
-  const bool h = lane & 16, m = lane & 8, l = lane & 4;
-  TV p[4], q[2];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) p[i] = (h ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h ? v[i] : v[i + 4], 16);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) q[i] = (m ? p[i + 2] : p[i]) + __shfl_xor_sync(0xffffffffu, m ? p[i] : p[i + 2], 8);
-  TV k = (l ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, l ? q[0] : q[1], 4);
-  k += __shfl_xor_sync(0xffffffffu, k, 2);
-  return k + __shfl_xor_sync(0xffffffffu, k, 1);
-}
-
 constexpr int kDotsGroup = 32;  // chunks whose partial sums one CTA adds before the last CTA does
 template <typename TV>
 constexpr int kDotsRows = sizeof(TV) == 4 ? 8 : 4;  // rows of u and w in a lane's registers
@@ -1297,10 +1282,9 @@ constexpr int kDotsRows = sizeof(TV) == 4 ? 8 : 4;  // rows of u and w in a lane
 // warp passes over all the basis vectors, the next one's loads in flight while one is summed, so the warps
 // stay balanced at every j and nothing waits for a staged copy.  The partial sums of kDotsGroup chunks are
 // added by the group's last CTA, those of the groups by the last CTA of all: a single CTA adding 1,003
-// partials of each of up to 100 sums took as long as the pass over the rows.  The rows of a warp (256) are
-// added in float32 as a tree, depth 13 (64 in sequence before), the rest in float64.  Every sum has a fixed
-// order (results do not depend on timing).  400,001 wires at one incidence, 37 steps: 5.6 ->
-// 3.7 ms; 24,535 wires at 181 incidences 2.6 -> 2.0 ms.
+// partials of each of up to 100 sums took as long as the pass over the rows.  In complex64 the rows of a warp
+// (256) are added in float32 or, in the steps before P.pair_steps, at most two rows in float32 and those sums
+// as error-free pairs; the rest in float64.  Every sum has a fixed order (results do not depend on timing).
 template <typename TV, typename TQ>
 __global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __restrict__ U,
                                                                          const cplx<TV>* __restrict__ Wv,
@@ -1316,76 +1300,81 @@ __global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __res
   constexpr int kWarps = kRows / 32, KR = kDotsRows<TV>;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  double* slot = reinterpret_cast<double*>(sm_raw);  // [j + 1][kWarps][4]
   const int64_t end = min(P.N, (int64_t)(blockIdx.x + 1) * P.chunk);
   const int64_t rn = (int64_t)r * P.N, vst = (int64_t)P.R * P.N;
   const float qsi = P.qsi;
-  bool first = true;
-  for (int64_t n0 = (int64_t)blockIdx.x * P.chunk; n0 < end; n0 += KR * kRows, first = false) {
-    const int64_t n = n0 + threadIdx.x;
-    const int left = n < end ? (int)min((int64_t)KR, (end - n + kRows - 1) / kRows) : 0;  // rows of this thread
-    cplx<TV> x[KR], y[KR];
-#pragma unroll
-    for (int k = 0; k < KR; ++k) {
-      x[k] = y[k] = mkc<TV>(0, 0);
-      if (k < left) {
-        x[k] = U[rn + n + kRows * k];
-        if (!closing) y[k] = Wv[rn + n + kRows * k];
-      }
-    }
-    const TQ* vq = V + rn + n;
-    auto load = [&](cplx<TV> (&v)[KR]) {
-#pragma unroll
-      for (int k = 0; k < KR; ++k) v[k] = k < left ? QStore<TV, TQ>::ld(vq + kRows * k, qsi) : mkc<TV>(0, 0);
-      vq += vst;
-    };
-    auto dot = [&](const cplx<TV> (&v)[KR], TV* o) {
-      cplx<TV> a = mkc<TV>(0, 0), b = mkc<TV>(0, 0);
-#pragma unroll
-      for (int k = 0; k < KR; ++k) {
-        a.re = fma(v[k].re, x[k].re, fma(v[k].im, x[k].im, a.re));
-        a.im = fma(v[k].re, x[k].im, fma(-v[k].im, x[k].re, a.im));
-        b.re = fma(v[k].re, y[k].re, fma(v[k].im, y[k].im, b.re));
-        b.im = fma(v[k].re, y[k].im, fma(-v[k].im, y[k].re, b.im));
-      }
-      o[0] = a.re;
-      o[1] = a.im;
-      o[2] = b.re;
-      o[3] = b.im;
-    };
-    cplx<TV> v0[KR], v1[KR];
-    if (j > 0) load(v0);
-    for (int i = 0; i <= j; i += 2) {  // the j-th vector is u itself
-      TV d[8];
-      if (i + 1 < j) load(v1);
-      if (i < j)
-        dot(v0, d);
-      else
-        dot(x, d);
-      if (i + 2 < j) load(v0);
-      if (i + 1 < j)
-        dot(v1, d + 4);
-      else if (i + 1 == j)
-        dot(x, d + 4);
-      else
-        d[4] = d[5] = d[6] = d[7] = TV(0);
-      const double t = (double)warp_sum8<TV>(d, lane);
-      const int ii = i + (lane >> 4);
-      if ((lane & 3) == 0 && ii <= j) {
-        double* s = slot + (ii * kWarps + wp) * 4 + ((lane >> 2) & 3);  // this lane's own over all the pieces
-        *s = first ? t : *s + t;
-      }
-    }
-  }
-  __syncthreads();
   // partials laid out [r][2 i + k][chunk]: a group of chunks is one contiguous run
   c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
-  for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
-    const double* sl = slot + (e >> 1) * (kWarps * 4) + 2 * (e & 1);
-    c128 t = mkc(0.0, 0.0);
+  auto pass = [&](auto none) {
+    using Sum = decltype(none);
+    using Acc = std::conditional_t<std::is_same<Sum, float>::value, double, Sum>;  // over pieces and warps
+    Acc* slot = reinterpret_cast<Acc*>(sm_raw);  // [j + 1][kWarps][4]
+    bool first = true;
+    for (int64_t n0 = (int64_t)blockIdx.x * P.chunk; n0 < end; n0 += KR * kRows, first = false) {
+      const int64_t n = n0 + threadIdx.x;
+      const int left = n < end ? (int)min((int64_t)KR, (end - n + kRows - 1) / kRows) : 0;  // rows of this thread
+      cplx<TV> x[KR], y[KR];
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) t = t + mkc(sl[4 * w], sl[4 * w + 1]);
-    part[(int64_t)e * P.nchunk + blockIdx.x] = t;
+      for (int k = 0; k < KR; ++k) {
+        x[k] = y[k] = mkc<TV>(0, 0);
+        if (k < left) {
+          x[k] = U[rn + n + kRows * k];
+          if (!closing) y[k] = Wv[rn + n + kRows * k];
+        }
+      }
+      const TQ* vq = V + rn + n;
+      auto load = [&](cplx<TV> (&v)[KR]) {
+#pragma unroll
+        for (int k = 0; k < KR; ++k) v[k] = k < left ? QStore<TV, TQ>::ld(vq + kRows * k, qsi) : mkc<TV>(0, 0);
+        vq += vst;
+      };
+      auto dot = [&](const cplx<TV> (&v)[KR], Sum* o) {
+        lane_dot(v, x, o);
+        lane_dot(v, y, o + 2);
+      };
+      cplx<TV> v0[KR], v1[KR];
+      if (j > 0) load(v0);
+      for (int i = 0; i <= j; i += 2) {  // the j-th vector is u itself
+        Sum d[8];
+        if (i + 1 < j) load(v1);
+        if (i < j)
+          dot(v0, d);
+        else
+          dot(x, d);
+        if (i + 2 < j) load(v0);
+        if (i + 1 < j)
+          dot(v1, d + 4);
+        else if (i + 1 == j)
+          dot(x, d + 4);
+        else
+          d[4] = d[5] = d[6] = d[7] = Sum{};
+        const Acc t = (Acc)warp_sum8(d, lane);
+        const int ii = i + (lane >> 4);
+        if ((lane & 3) == 0 && ii <= j) {
+          Acc* s = slot + (ii * kWarps + wp) * 4 + ((lane >> 2) & 3);  // this lane's own over all the pieces
+          *s = first ? t : *s + t;
+        }
+      }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
+      const Acc* sl = slot + (e >> 1) * (kWarps * 4) + 2 * (e & 1);
+      Acc re = sl[0], im = sl[1];
+#pragma unroll
+      for (int w = 1; w < kWarps; ++w) {
+        re = re + sl[4 * w];
+        im = im + sl[4 * w + 1];
+      }
+      part[(int64_t)e * P.nchunk + blockIdx.x] = mkc(widen(re), widen(im));
+    }
+  };
+  if constexpr (sizeof(TV) == 4) {
+    if (j < P.pair_steps)
+      pass(FPair{});
+    else
+      pass(0.f);
+  } else {
+    pass(0.0);
   }
   if (P.ngroup <= 1) {
     if (!last_cta(P, r)) return;
@@ -1421,7 +1410,7 @@ __global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __res
     for (int u = 0; u < EB; u += 4) {
       const double d[8] = {v[u].x,     v[u].y,     v[u + 1].x, v[u + 1].y,
                            v[u + 2].x, v[u + 2].y, v[u + 3].x, v[u + 3].y};
-      const double t = warp_sum8<double>(d, lane);
+      const double t = warp_sum8(d, lane);
       const int e = e0 + (u + (lane >> 3)) * kWarps;
       if ((lane & 3) == 0 && e < 2 * (j + 1))
         reinterpret_cast<double*>(gpart + (int64_t)e * P.ngroup + gr)[(lane >> 2) & 1] = t;
@@ -1662,6 +1651,23 @@ __global__ void k_rowwire(int64_t nw, const int64_t* __restrict__ off, Layout la
   }
 }
 
+// Complex64 steps whose dots add the lanes' float32 sums as pairs.  A lane adds n rows in float32, and the 32
+// lanes' sums added in float32 too leave a sum of values of one sign (|u|^2) a variance of n^2 + 94.5 n,
+// where strands of m rows, each widened to float64 by itself, leave m^2 (in the same units).  With eight
+// strands a lane in step 0, four in step 1, and so on to one, m is eight rows of a long chunk in step 0
+// and 64 from step 7 on: short sums need the pairs at n = 8 in two steps of a large system and in every step of
+// a small one, later sums do not.  Pairs in every step cost 400,001 wires at one incidence 0.45 ms of 14.5 ms.
+int dots_pair_steps(int64_t N, int R, int64_t nsm, int64_t chunk, int restart) {
+  const int64_t strands = std::min<int64_t>(2048, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, 4 * nsm), kRows) * kRows));
+  const int64_t n = std::min<int64_t>(kDotsRows<float>, ceil_div(std::min(chunk, N), kRows));
+  int j = 0;
+  for (; j <= restart; ++j) {
+    const int64_t m = ceil_div(ceil_div(std::min(strands, N), j < 7 ? 8 / (j + 1) : 1), 32);
+    if (m * m >= n * n + 95 * n) break;
+  }
+  return j;
+}
+
 // Restarted GMRES on A = I + E with E stored as TE.  With y_out the result stays in y-space
 // (*y_out = the workspace's y, no M^-1 and no statistics); otherwise x = M^-1 y goes to ctx->Xv.
 template <typename TV, typename TE, typename TQ = cplx<TV>>
@@ -1695,6 +1701,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   if (slots / R < 16) dchunk = std::min(dchunk, 4 * dpiece);
   P.chunk = (int)(ceil_div(std::max<int64_t>(dchunk, kRows), 32) * 32);
   P.nchunk = (int)ceil_div(N, P.chunk);
+  P.pair_steps = dots_pair_steps(N, R, nsm, P.chunk, restart);
   P.ngroup = P.nchunk > 2 * kDotsGroup ? (int)ceil_div(P.nchunk, kDotsGroup) : 1;
   const int R1 = restart + 1;
   // The workspace persists across solves of the same size, so buffer addresses (and the captured

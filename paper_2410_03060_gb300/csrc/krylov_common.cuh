@@ -44,6 +44,7 @@ struct KPtr {
   unsigned* gcounter; // [R][ngroup] CTAs of the current pass that have arrived
   double* partn;      // [R][nchunk]
   int ngroup;         // groups of chunks (1: the partials are added without groups)
+  int pair_steps;     // complex64 steps whose dots add the lanes' float32 sums as pairs
   int R, restart, nchunk, chunk;  // rows per CTA of the dots and cycle-start kernels
   int nuchunk, uchunk;             // rows per CTA of the update
   int max_iter;
