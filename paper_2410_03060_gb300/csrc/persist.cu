@@ -458,7 +458,7 @@ __device__ void p_product_columns(int mode, const PArgs& a, const ESlice<TV, TE>
 // Rows of the CTA times A = I + E for the R right-hand sides of `src`.
 // mode 0 (Arnoldi): ws = u + E u for the pending vector u (own rows in ys, all rows in src).
 // mode 1 (residual): ys = W = B - (Y + E Y), squared norms to partn.
-template <typename TV, typename TE, int RB>
+template <typename TV, typename TE, int RB, bool WIDE>
 __device__ void p_product(int mode, const PArgs& a, const ESlice<TV, TE>& S, const cplx<TV>* __restrict__ src,
                           cplx<TV>* ys, cplx<TV>* ws, int cnt, int64_t n0, const int* act,
                           const cplx<TV>* __restrict__ B, cplx<TV>* __restrict__ W, TV (*red)[RB]) {
@@ -496,14 +496,14 @@ __device__ void p_product(int mode, const PArgs& a, const ESlice<TV, TE>& S, con
     }
     __syncthreads();
   }
-  if constexpr (RB == 1) {
-    if (a.wide == 2) {
-      p_product_columns<TV, TE>(mode, a, S, src, ys, ws, cnt, n0, on[0], B, W, nrm[0]);
-      if (mode == 1) p_norm_partials<TV, RB>(nrm, R, a.G, (TV*)a.partn, red);
-      return;
+  if constexpr (WIDE) {
+    if constexpr (RB == 1) {
+      if (a.wide == 2) {
+        p_product_columns<TV, TE>(mode, a, S, src, ys, ws, cnt, n0, on[0], B, W, nrm[0]);
+        if (mode == 1) p_norm_partials<TV, RB>(nrm, R, a.G, (TV*)a.partn, red);
+        return;
+      }
     }
-  }
-  if (!S.xg && a.wide) {
     // Long rows streamed from global memory (entire coupling: 5,128 entries a row at 1,000 wires,
     // 210 MB of E per product): a warp per row, eight coalesced loads of E in flight per lane.
     // Bound by HBM.  Four lanes per row read 32-byte pieces of eight rows: 0.63 ms per product
@@ -658,7 +658,10 @@ __device__ void p_residual_zero(const PArgs& a, cplx<TV>* ys, int cnt, int64_t n
   p_norm_partials<TV, RB>(nrm, R, a.G, (TV*)a.partn, red);
 }
 
-template <typename TV, typename TE, int RB>
+// WIDE: the form for long rows of E in global memory (PArgs::wide).  A kernel of its own: its loads in flight
+// take registers that the other form's steps spilled (209 unknowns, one incidence: the solve 165 us in one
+// kernel, 152 us so; 1,532 unknowns in complex128, four incidences 2.15 and 2.10 ms).
+template <typename TV, typename TE, int RB, bool WIDE>
 __global__ void __launch_bounds__(kPT, 1) k_gmres_persist(PArgs a) {
   using C = cplx<TV>;
   const KPtr& P = a.P;
@@ -794,7 +797,7 @@ __global__ void __launch_bounds__(kPT, 1) k_gmres_persist(PArgs a) {
     if (first && a.y_zero)
       p_residual_zero<TV, RB>(a, ys, cnt, n0, (C*)a.B, Y, W, red);
     else
-      p_product<TV, TE, RB>(1, a, S, Y, ys, ws, cnt, n0, act, B, W, red);
+      p_product<TV, TE, RB, WIDE>(1, a, S, Y, ys, ws, cnt, n0, act, B, W, red);
     if (!(ok = grid_sync(a.sync, a.arrivals, &s_epoch, &s_ok))) break;
     // ---- start of a cycle (every CTA)
     if (wp < R) {
@@ -832,7 +835,7 @@ __global__ void __launch_bounds__(kPT, 1) k_gmres_persist(PArgs a) {
       const int j = s_j;
       const bool closing = j >= s_jmax;
       // A: w = A u_j on own rows, partial dots
-      if (!closing) p_product<TV, TE, RB>(0, a, S, W, ys, ws, cnt, n0, act, B, W, red);
+      if (!closing) p_product<TV, TE, RB, WIDE>(0, a, S, W, ys, ws, cnt, n0, act, B, W, red);
       __syncthreads();
       p_dots2<TV>(V, ys, ws, a.rows, cnt, R, R1, j, G, act, closing, part1, part2);
       if (!(ok = grid_sync(a.sync, a.arrivals, &s_epoch, &s_ok))) break;
@@ -1043,9 +1046,10 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   const int R = P.R, restart = P.restart;
   const int64_t N = P.N;
   const int ctas = ctx->persist_ctas > 0 ? std::min(ctx->persist_ctas, std::max(ctx->nsm, 1)) : std::max(ctx->nsm, 1);
-  // Rows per CTA.  A multiple of 32 where a CTA's rows are few and short (fewer CTAs, cheaper
-  // barriers and sums); with long rows streamed from global memory every SM has to take its share
-  // (5,133 rows: 151 CTAs of 34 rows instead of 81 of 64).
+  // Rows per CTA.  A multiple of 32 where rows are short (fewer CTAs, cheaper barriers and sums); with long
+  // rows every SM takes its share (5,133 rows: 151 CTAs of 34 rows instead of 81 of 64), also where E then
+  // lies in shared memory: entire coupling by two and by 32 rows, one incidence, 147 to 507 rows within 4 % of
+  // one another; four incidences, 209 rows 0.21 and 0.34 ms.
   const bool wide = ctx->offd.nval >= kPersistWideRow * N;
   const int64_t rgran = wide ? 2 : 32;
   const int prows = (int)(ceil_div(ceil_div(std::max<int64_t>(N, 1), ctas), rgran) * rgran);
@@ -1054,10 +1058,11 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
     return SWM_OK;
   const int G = (int)ceil_div(N, prows);
   const int RB = R == 1 ? 1 : kPersistMaxR;
-  const void* fn = R == 1 ? (const void*)k_gmres_persist<TV, TE, 1> : (const void*)k_gmres_persist<TV, TE, kPersistMaxR>;
+  const void* fn = R == 1 ? (const void*)k_gmres_persist<TV, TE, 1, false>
+                          : (const void*)k_gmres_persist<TV, TE, kPersistMaxR, false>;
   size_t static_smem = 0;
   SWM_CK(allow_max_dyn_smem(fn, ctx->smem_optin, &static_smem));
-  const size_t limit = (size_t)std::max(0, ctx->smem_optin - (int)static_smem - 1024);
+  size_t limit = (size_t)std::max(0, ctx->smem_optin - (int)static_smem - 1024);
   const size_t cb = sizeof(cplx<TV>), eb = sizeof(TE);
   // V in shared memory when it fits (it is read twice a step); then as large an E slice as
   // the rest holds (column map + gathered vector about a third of the E entries: the rows of a
@@ -1077,6 +1082,13 @@ int gmres_persistent(swm_ctx* ctx, const KPtr& P, const PBuffers& Bf, int max_it
   const size_t pw = cb * kPWarps * (size_t)prows;
   const bool columns = wide && !esm && R == 1 && prows <= kPersistColumnRows && smem + pw <= limit;
   if (columns) smem += pw;
+  if (wide && !esm) {
+    fn = R == 1 ? (const void*)k_gmres_persist<TV, TE, 1, true>
+                : (const void*)k_gmres_persist<TV, TE, kPersistMaxR, true>;
+    size_t wide_static = 0;
+    SWM_CK(allow_max_dyn_smem(fn, ctx->smem_optin, &wide_static));
+    if (wide_static > static_smem) limit -= std::min(limit, wide_static - static_smem);
+  }
   if (smem > limit) return SWM_OK;
   int occ = 0;
   SWM_CK(occupancy_cached(fn, kPT, smem, &occ));
