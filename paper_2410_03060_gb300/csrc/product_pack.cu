@@ -406,7 +406,13 @@ int ensure_row_order(swm_ctx* ctx) {
   SWM_CK(cudaStreamIsCapturing(ctx->stream, &cs));
   if (cs != cudaStreamCaptureStatusNone) return SWM_OK;
   int32_t* w = nullptr;
-  SWM_TRY(dalloc(ctx, ctx->pattern_bufs, (void**)&w, sizeof(int32_t) * ctx->nw));
+  const std::string err = ctx->err;
+  const int rc = dalloc(ctx, ctx->pattern_bufs, (void**)&w, sizeof(int32_t) * ctx->nw);
+  if (rc == SWM_ENOMEM) {  // the products run without it
+    ctx->err = err;
+    return SWM_OK;
+  }
+  if (rc < 0) return rc;
   k_pack_order<<<(unsigned)ceil_div(ctx->nw, kPackWin), 1024, 0, ctx->stream>>>(ctx->nw, ctx->offd, ctx->off, nullptr,
                                                                                nullptr, w);
   SWM_LAUNCHED();
