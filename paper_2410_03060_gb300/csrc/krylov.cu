@@ -1272,116 +1272,20 @@ __device__ void dots_tail(const KPtr& P, int j, int r, bool closing, const c128*
 }
 
 constexpr int kDotsGroup = 32;  // chunks whose partial sums one CTA adds before the last CTA does
-template <typename TV>
-constexpr int kDotsRows = sizeof(TV) == 4 ? 8 : 4;  // rows of u and w in a lane's registers
+constexpr int kDotsRows = 8;    // rows of u and w in a lane's registers
 
-// Dots of step j, one CTA per chunk of rows and right-hand side: for i < j the pairs
-// (q_i^H u, q_i^H w), and (|u|^2, u^H w), where u is the pending vector and w = A u; the closing
-// pass of a cycle (j = jmax, no product) takes only the first of each pair.  Bound by HBM (the basis is
-// read once; in float64 by its multiply-adds).  A lane keeps its rows of u and w in registers and every
-// warp passes over all the basis vectors, the next one's loads in flight while one is summed, so the warps
-// stay balanced at every j and nothing waits for a staged copy.  The partial sums of kDotsGroup chunks are
-// added by the group's last CTA, those of the groups by the last CTA of all: a single CTA adding 1,003
-// partials of each of up to 100 sums took as long as the pass over the rows.  In complex64 the rows of a warp
-// (256) are added in float32 or, in the steps before P.pair_steps, at most two rows in float32 and those sums
-// as error-free pairs; the rest in float64.  Every sum has a fixed order (results do not depend on timing).
-template <typename TV, typename TQ>
-__global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __restrict__ U,
-                                                                         const cplx<TV>* __restrict__ Wv,
-                                                                         const TQ* __restrict__ V) {
-  if (P.st->cycle_done) return;
-  const int j = P.st->j, r = blockIdx.y;
-  const bool closing = j >= P.st->jmax;
-  if (!P.active[r]) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) step_arrive(P, j, closing);
-    return;
-  }
-  const int R1 = P.restart + 1;
-  constexpr int kWarps = kRows / 32, KR = kDotsRows<TV>;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int64_t end = min(P.N, (int64_t)(blockIdx.x + 1) * P.chunk);
-  const int64_t rn = (int64_t)r * P.N, vst = (int64_t)P.R * P.N;
-  const float qsi = P.qsi;
-  // partials laid out [r][2 i + k][chunk]: a group of chunks is one contiguous run
-  c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
-  auto pass = [&](auto none) {
-    using Sum = decltype(none);
-    using Acc = std::conditional_t<std::is_same<Sum, float>::value, double, Sum>;  // over pieces and warps
-    Acc* slot = reinterpret_cast<Acc*>(sm_raw);  // [j + 1][kWarps][4]
-    bool first = true;
-    for (int64_t n0 = (int64_t)blockIdx.x * P.chunk; n0 < end; n0 += KR * kRows, first = false) {
-      const int64_t n = n0 + threadIdx.x;
-      const int left = n < end ? (int)min((int64_t)KR, (end - n + kRows - 1) / kRows) : 0;  // rows of this thread
-      cplx<TV> x[KR], y[KR];
-#pragma unroll
-      for (int k = 0; k < KR; ++k) {
-        x[k] = y[k] = mkc<TV>(0, 0);
-        if (k < left) {
-          x[k] = U[rn + n + kRows * k];
-          if (!closing) y[k] = Wv[rn + n + kRows * k];
-        }
-      }
-      const TQ* vq = V + rn + n;
-      auto load = [&](cplx<TV> (&v)[KR]) {
-#pragma unroll
-        for (int k = 0; k < KR; ++k) v[k] = k < left ? QStore<TV, TQ>::ld(vq + kRows * k, qsi) : mkc<TV>(0, 0);
-        vq += vst;
-      };
-      auto dot = [&](const cplx<TV> (&v)[KR], Sum* o) {
-        lane_dot(v, x, o);
-        lane_dot(v, y, o + 2);
-      };
-      cplx<TV> v0[KR], v1[KR];
-      if (j > 0) load(v0);
-      for (int i = 0; i <= j; i += 2) {  // the j-th vector is u itself
-        Sum d[8];
-        if (i + 1 < j) load(v1);
-        if (i < j)
-          dot(v0, d);
-        else
-          dot(x, d);
-        if (i + 2 < j) load(v0);
-        if (i + 1 < j)
-          dot(v1, d + 4);
-        else if (i + 1 == j)
-          dot(x, d + 4);
-        else
-          d[4] = d[5] = d[6] = d[7] = Sum{};
-        const Acc t = (Acc)warp_sum8(d, lane);
-        const int ii = i + (lane >> 4);
-        if ((lane & 3) == 0 && ii <= j) {
-          Acc* s = slot + (ii * kWarps + wp) * 4 + ((lane >> 2) & 3);  // this lane's own over all the pieces
-          *s = first ? t : *s + t;
-        }
-      }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
-      const Acc* sl = slot + (e >> 1) * (kWarps * 4) + 2 * (e & 1);
-      Acc re = sl[0], im = sl[1];
-#pragma unroll
-      for (int w = 1; w < kWarps; ++w) {
-        re = re + sl[4 * w];
-        im = im + sl[4 * w + 1];
-      }
-      part[(int64_t)e * P.nchunk + blockIdx.x] = mkc(widen(re), widen(im));
-    }
-  };
-  if constexpr (sizeof(TV) == 4) {
-    if (j < P.pair_steps)
-      pass(FPair{});
-    else
-      pass(0.f);
-  } else {
-    pass(0.0);
-  }
+// The end of a dots CTA whose partial sums are in `part`: the last CTA of a group of kDotsGroup chunks adds
+// the group's partials, the last group's CTA the groups', and goes on to the step's tail.  A single CTA
+// adding 1,003 partials of each of up to 100 sums took as long as the pass over the rows.
+template <typename TV>
+__device__ __forceinline__ void dots_end(const KPtr& P, int j, int r, bool closing, const c128* part) {
+  constexpr int kWarps = kRows / 32;
+  const int R1 = P.restart + 1, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (P.ngroup <= 1) {
     if (!last_cta(P, r)) return;
     dots_tail<TV>(P, j, r, closing, part, P.nchunk);
     return;
   }
-  // the last CTA of the group adds the group's partials, then the last group's CTA goes on
   __shared__ bool last;
   const int gr = blockIdx.x / kDotsGroup;
   const int c0 = gr * kDotsGroup, gn = min(kDotsGroup, P.nchunk - c0);
@@ -1423,6 +1327,202 @@ __global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const cplx<TV>* __res
   if (!last) return;
   __threadfence();
   dots_tail<TV>(P, j, r, closing, gpart, P.ngroup);
+}
+
+// Dots of step j, one CTA per chunk of rows and right-hand side: for i < j the pairs
+// (q_i^H u, q_i^H w), and (|u|^2, u^H w), where u is the pending vector and w = A u; the closing
+// pass of a cycle (j = jmax, no product) takes only the first of each pair.
+//
+// Complex64 (and a half-precision basis of fewer than kStagedRows rows in all).  Bound by HBM (the basis is
+// read once).  A lane keeps its rows of u and w in registers and every warp passes over all the basis vectors,
+// the next one's loads in flight while one is summed, so the warps stay balanced at every j and nothing waits
+// for a staged copy.  The rows of a warp (256) are added in float32 or, in the steps before P.pair_steps, at
+// most two rows in float32 and those sums as error-free pairs; the rest in float64.  Every sum has a fixed
+// order (results do not depend on timing).
+template <typename TQ>
+__global__ void __launch_bounds__(kRows, 2) k_dots(KPtr P, const c64* __restrict__ U, const c64* __restrict__ Wv,
+                                                   const TQ* __restrict__ V) {
+  if (P.st->cycle_done) return;
+  const int j = P.st->j, r = blockIdx.y;
+  const bool closing = j >= P.st->jmax;
+  if (!P.active[r]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) step_arrive(P, j, closing);
+    return;
+  }
+  const int R1 = P.restart + 1;
+  constexpr int kWarps = kRows / 32, KR = kDotsRows;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int64_t end = min(P.N, (int64_t)(blockIdx.x + 1) * P.chunk);
+  const int64_t rn = (int64_t)r * P.N, vst = (int64_t)P.R * P.N;
+  const float qsi = P.qsi;
+  // partials laid out [r][2 i + k][chunk]: a group of chunks is one contiguous run
+  c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
+  auto pass = [&](auto none) {
+    using Sum = decltype(none);
+    using Acc = std::conditional_t<std::is_same<Sum, float>::value, double, Sum>;  // over pieces and warps
+    Acc* slot = reinterpret_cast<Acc*>(sm_raw);  // [j + 1][kWarps][4]
+    bool first = true;
+    for (int64_t n0 = (int64_t)blockIdx.x * P.chunk; n0 < end; n0 += KR * kRows, first = false) {
+      const int64_t n = n0 + threadIdx.x;
+      const int left = n < end ? (int)min((int64_t)KR, (end - n + kRows - 1) / kRows) : 0;  // rows of this thread
+      c64 x[KR], y[KR];
+#pragma unroll
+      for (int k = 0; k < KR; ++k) {
+        x[k] = y[k] = mkc<float>(0, 0);
+        if (k < left) {
+          x[k] = U[rn + n + kRows * k];
+          if (!closing) y[k] = Wv[rn + n + kRows * k];
+        }
+      }
+      const TQ* vq = V + rn + n;
+      auto load = [&](c64 (&v)[KR]) {
+#pragma unroll
+        for (int k = 0; k < KR; ++k) v[k] = k < left ? QStore<float, TQ>::ld(vq + kRows * k, qsi) : mkc<float>(0, 0);
+        vq += vst;
+      };
+      auto dot = [&](const c64 (&v)[KR], Sum* o) {
+        lane_dot(v, x, o);
+        lane_dot(v, y, o + 2);
+      };
+      c64 v0[KR], v1[KR];
+      if (j > 0) load(v0);
+      for (int i = 0; i <= j; i += 2) {  // the j-th vector is u itself
+        Sum d[8];
+        if (i + 1 < j) load(v1);
+        if (i < j)
+          dot(v0, d);
+        else
+          dot(x, d);
+        if (i + 2 < j) load(v0);
+        if (i + 1 < j)
+          dot(v1, d + 4);
+        else if (i + 1 == j)
+          dot(x, d + 4);
+        else
+          d[4] = d[5] = d[6] = d[7] = Sum{};
+        const Acc t = (Acc)warp_sum8(d, lane);
+        const int ii = i + (lane >> 4);
+        if ((lane & 3) == 0 && ii <= j) {
+          Acc* s = slot + (ii * kWarps + wp) * 4 + ((lane >> 2) & 3);  // this lane's own over all the pieces
+          *s = first ? t : *s + t;
+        }
+      }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
+      const Acc* sl = slot + (e >> 1) * (kWarps * 4) + 2 * (e & 1);
+      Acc re = sl[0], im = sl[1];
+#pragma unroll
+      for (int w = 1; w < kWarps; ++w) {
+        re = re + sl[4 * w];
+        im = im + sl[4 * w + 1];
+      }
+      part[(int64_t)e * P.nchunk + blockIdx.x] = mkc(widen(re), widen(im));
+    }
+  };
+  if (j < P.pair_steps)
+    pass(FPair{});
+  else
+    pass(0.f);
+  dots_end<float>(P, j, r, closing, part);
+}
+
+// The same in float64, and for a half-precision basis of kStagedRows rows and more: the chunk's rows of u and
+// w are staged in shared memory; the warps take (i, row slice) items, q_j standing for u itself, with the rows
+// split into S slices while j + 1 < 8 so that every warp streams, and eight loads in flight per lane.  Slice
+// sums are added in a fixed order.  A lane adds up to 64 rows before a sum costs its warp float64 additions,
+// which set the time in float64: with four rows in registers 20,000 wires at 60 incidences took 86.7 ms, so
+// 74.0, 1,000 wires at one 1.04 and 0.70 ms.  The bfloat16 solve's cycles are short, where the registers' form
+// waits for u and w more than it reads the basis: 60,000 wires at 20 incidences 6.2 and 3.6 ms, 120,000 at one
+// (615,781 rows) 1.79 and 1.57 ms, 60,000 at one 1.34 and 1.42 ms.
+constexpr int64_t kStagedRows = 1 << 19;
+template <typename TV, typename TQ>
+__global__ void __launch_bounds__(kRows) k_dots_staged(KPtr P, const cplx<TV>* __restrict__ U,
+                                                       const cplx<TV>* __restrict__ Wv, const TQ* __restrict__ V) {
+  if (P.st->cycle_done) return;
+  const int j = P.st->j, r = blockIdx.y;
+  const bool closing = j >= P.st->jmax;
+  if (!P.active[r]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) step_arrive(P, j, closing);
+    return;
+  }
+  const int R1 = P.restart + 1;
+  constexpr int kWarps = kRows / 32;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int64_t n0 = (int64_t)blockIdx.x * P.chunk;
+  const int cnt = (int)min((int64_t)P.chunk, P.N - n0);
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  cplx<TV>* u_sm = reinterpret_cast<cplx<TV>*>(sm_raw);  // [chunk]
+  cplx<TV>* w_sm = u_sm + P.chunk;                       // [chunk]
+  __shared__ c128 slot[2 * (SWM_MAX_RESTART + 1)];
+  const cplx<TV>* u = U + (int64_t)r * P.N + n0;
+  const cplx<TV>* w = Wv + (int64_t)r * P.N + n0;
+  for (int t = threadIdx.x; t < cnt; t += kRows) {
+    u_sm[t] = u[t];
+    if (!closing) w_sm[t] = w[t];
+  }
+  __syncthreads();
+  const int S = j + 1 >= kWarps ? 1 : kWarps / (j + 1);  // row slices per i
+  const int len = ((cnt + S - 1) / S + 31) / 32 * 32;
+  for (int item = wp; item < (j + 1) * S; item += kWarps) {
+    const int i = item / S, sl = item % S;
+    const int lo = sl * len, hi = min(cnt, lo + len);
+    // q_i from the basis, or (i == j) the pending vector u itself from shared memory; a basis in
+    // the vector type is read through one pointer, a half-precision one converted on load
+    constexpr bool full = std::is_same<TQ, cplx<TV>>::value;
+    const TQ* vq = V + ((int64_t)i * P.R + r) * P.N + n0;  // i <= j <= restart: inside the basis
+    const cplx<TV>* vi = full ? (i < j ? reinterpret_cast<const cplx<TV>*>(vq) : u_sm) : u_sm;
+    const bool own = i >= j;
+    const float qsi = P.qsi;
+    auto ldv = [&](int t) -> cplx<TV> {
+      if constexpr (full) return vi[t];
+      else return own ? u_sm[t] : QStore<TV, TQ>::ld(vq + t, qsi);
+    };
+    cplx<TV> a = mkc<TV>(0, 0), b = mkc<TV>(0, 0);
+    int t = lo + lane;
+    for (; t + 224 < hi; t += 256) {
+      cplx<TV> v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = ldv(t + 32 * k);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const cplx<TV> x = u_sm[t + 32 * k];
+        a.re = fma(v[k].re, x.re, fma(v[k].im, x.im, a.re));
+        a.im = fma(v[k].re, x.im, fma(-v[k].im, x.re, a.im));
+        if (!closing) {
+          const cplx<TV> y = w_sm[t + 32 * k];
+          b.re = fma(v[k].re, y.re, fma(v[k].im, y.im, b.re));
+          b.im = fma(v[k].re, y.im, fma(-v[k].im, y.re, b.im));
+        }
+      }
+    }
+    for (; t < hi; t += 32) {
+      const cplx<TV> v = ldv(t), x = u_sm[t];
+      a.re = fma(v.re, x.re, fma(v.im, x.im, a.re));
+      a.im = fma(v.re, x.im, fma(-v.im, x.re, a.im));
+      if (!closing) {
+        const cplx<TV> y = w_sm[t];
+        b.re = fma(v.re, y.re, fma(v.im, y.im, b.re));
+        b.im = fma(v.re, y.im, fma(-v.im, y.re, b.im));
+      }
+    }
+    const double ar = warp_sum((double)a.re), ai = warp_sum((double)a.im);
+    const double br = warp_sum((double)b.re), bi = warp_sum((double)b.im);
+    if (lane == 0) {
+      slot[2 * item] = mkc(ar, ai);
+      slot[2 * item + 1] = mkc(br, bi);
+    }
+  }
+  __syncthreads();
+  c128* part = P.part + (int64_t)r * 2 * R1 * P.nchunk;
+  for (int e = threadIdx.x; e < 2 * (j + 1); e += kRows) {
+    const int i = e >> 1, k = e & 1;
+    c128 v = slot[2 * (i * S) + k];
+    for (int sl = 1; sl < S; ++sl) v = v + slot[2 * (i * S + sl) + k];
+    part[(int64_t)e * P.nchunk + blockIdx.x] = v;
+  }
+  dots_end<TV>(P, j, r, closing, part);
 }
 
 // Update of step j (after its dots): q_j = (u - Q s) / rho goes to V_j and the next pending vector
@@ -1659,7 +1759,7 @@ __global__ void k_rowwire(int64_t nw, const int64_t* __restrict__ off, Layout la
 // a small one, later sums do not.  Pairs in every step cost 400,001 wires at one incidence 0.45 ms of 14.5 ms.
 int dots_pair_steps(int64_t N, int R, int64_t nsm, int64_t chunk, int restart) {
   const int64_t strands = std::min<int64_t>(2048, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, 4 * nsm), kRows) * kRows));
-  const int64_t n = std::min<int64_t>(kDotsRows<float>, ceil_div(std::min(chunk, N), kRows));
+  const int64_t n = std::min<int64_t>(kDotsRows, ceil_div(std::min(chunk, N), kRows));
   int j = 0;
   for (; j <= restart; ++j) {
     const int64_t m = ceil_div(ceil_div(std::min(strands, N), j < 7 ? 8 / (j + 1) : 1), 32);
@@ -1687,19 +1787,24 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   P.max_iter = max_iter;
   P.qs = kFullBasis ? 1.f : (float)std::sqrt((double)std::max<int64_t>(1, N));
   P.qsi = 1.f / P.qs;
-  // rows per CTA of the Gram-Schmidt kernels: the update about 16 CTAs per SM over all right-hand
-  // sides, at most kMaxChunk; the dots one wave of CTAs (fewest partial sums), or, where that would leave
-  // a right-hand side fewer than 16 CTAs, up to four pieces per CTA in several waves; in float64 one piece
-  // per CTA (adding the next piece's sums would cost float64 instructions, which set the time there)
+  // rows per CTA of the Gram-Schmidt kernels: the update about 16 CTAs per SM over all right-hand sides and
+  // the staged dots about 4, at most kMaxChunk; the other dots one wave of CTAs (fewest partial sums), or, where
+  // that would leave a right-hand side fewer than 16 CTAs, up to four pieces per CTA in several waves
   const int64_t nsm = std::max(ctx->nsm, 1);
-  P.uchunk = (int)std::min<int64_t>(kMaxChunk, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, 16 * nsm), kRows) * kRows));
+  auto rows_per_cta = [&](int64_t per_sm) {
+    return (int)std::min<int64_t>(kMaxChunk, std::max<int64_t>(kRows, ceil_div(ceil_div(N * R, per_sm * nsm), kRows) * kRows));
+  };
+  P.uchunk = rows_per_cta(16);
   P.nuchunk = (int)ceil_div(N, P.uchunk);
-  constexpr int64_t dpiece = kDotsRows<TV> * kRows;
-  const int64_t slots = 2 * nsm;
-  int64_t dchunk = ceil_div(N, std::max<int64_t>(1, slots / R));
-  if (sizeof(TV) == 8) dchunk = std::min(dchunk, dpiece);
-  if (slots / R < 16) dchunk = std::min(dchunk, 4 * dpiece);
-  P.chunk = (int)(ceil_div(std::max<int64_t>(dchunk, kRows), 32) * 32);
+  const bool staged = sizeof(TV) == 8 || (!kFullBasis && N * R >= kStagedRows);
+  if (staged) {
+    P.chunk = rows_per_cta(4);
+  } else {
+    const int64_t slots = 2 * nsm;
+    int64_t dchunk = ceil_div(N, std::max<int64_t>(1, slots / R));
+    if (slots / R < 16) dchunk = std::min<int64_t>(dchunk, 4 * kDotsRows * kRows);
+    P.chunk = (int)(ceil_div(std::max<int64_t>(dchunk, kRows), 32) * 32);
+  }
   P.nchunk = (int)ceil_div(N, P.chunk);
   P.pair_steps = dots_pair_steps(N, R, nsm, P.chunk, restart);
   P.ngroup = P.nchunk > 2 * kDotsGroup ? (int)ceil_div(P.nchunk, kDotsGroup) : 1;
@@ -1931,7 +2036,11 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
       SWM_TRY(allow_wm<TE>(ctx));
     }
   }
-  const size_t dots_smem = sizeof(double) * 4 * (kRows / 32) * (size_t)R1;  // at most 33 KB
+  // the registers' form: at most 33 KB of sums; the staged form: the chunk's rows of u and w
+  const size_t dots_smem =
+      staged ? 2 * sizeof(cplx<TV>) * (size_t)P.chunk : sizeof(double) * 4 * (kRows / 32) * (size_t)R1;
+  if constexpr (sizeof(TV) == 8)  // float32: 32 KB
+    SWM_CK(allow_max_dyn_smem((const void*)k_dots_staged<TV, TQ>, ctx->smem_optin));
   // back substitution stages the triangle in shared memory when it fits
   size_t bs_smem = sizeof(c128) * (size_t)restart * restart;
   if (bs_smem > 160 * 1024) bs_smem = 0;
@@ -1948,7 +2057,14 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
       SWM_TRY(launch_product(s, rb));
       ctx->prof_end(SWM_K_APPLY);
       ctx->prof_begin(SWM_K_DOTS);
-      k_dots<TV, TQ><<<g_chunk, kRows, dots_smem, s>>>(P, U, Wv, V);
+      bool done = false;
+      if constexpr (sizeof(TV) == 8 || !kFullBasis) {
+        if (staged) k_dots_staged<TV, TQ><<<g_chunk, kRows, dots_smem, s>>>(P, U, Wv, V);
+        done = staged;
+      }
+      if constexpr (sizeof(TV) == 4) {
+        if (!done) k_dots<TQ><<<g_chunk, kRows, dots_smem, s>>>(P, U, Wv, V);
+      }
       ctx->prof_end(SWM_K_DOTS);
       SWM_LAUNCHED();
       ctx->prof_begin(SWM_K_UPDATE);
