@@ -180,7 +180,22 @@ __global__ void __launch_bounds__(kRows) k_spmv(KPtr P, const RowInfo* __restric
 // nothing was gained on a row per eight lanes.  CTAs of four warps at 64 registers (eight per SM, a few
 // spills) keep more of the short warps in flight; one column at a time in 48 registers was 2 % slower.
 // 400,001 wires, one incidence: the call 18.26 -> 17.25 ms.
+//
+// For complex64 systems of kOneWires wires and more, of kOneRowsPerWire rows a wire and more and of rows of at
+// most kOneMaxRow entries (use_spmv_one).  Elsewhere k_spmv, with more lanes in flight, is the faster one.  The
+// products of a solve there and here: 20,000 wires 0.42 and 0.47 ms, 20,000 of 15 rows 1.01 and 1.14 ms, 60,000
+// (of five rows, 48 entries a row) 1.41 and 1.40 ms, 120,000 1.18 and 0.96 ms; 90,000 of three rows 0.57 and 0.65 ms,
+// 400,000 of one row 0.63 and 1.56 ms; 120,000 of 160 entries a row 6.16 and 6.51 ms, 1,000 at entire coupling 4.1
+// and 7.2 ms; in bfloat16 60,000 wires 2.3 and 3.1 ms, in complex128 6.2 and 6.4 ms.
 constexpr int kOneThreads = 128;
+constexpr int64_t kOneWires = 50000;
+constexpr int64_t kOneRowsPerWire = 4;
+constexpr int64_t kOneMaxRow = 128;
+template <typename TV, typename TE>
+inline bool use_spmv_one(const swm_ctx* ctx) {
+  return std::is_same<TE, c64>::value && ctx->nw >= kOneWires && ctx->N >= kOneRowsPerWire * ctx->nw &&
+         ctx->offd.nval <= kOneMaxRow * ctx->N;
+}
 template <typename TV, typename TE, bool RES>
 __global__ void __launch_bounds__(kOneThreads, sizeof(TV) == 4 ? 8 : 4)
     k_spmv_one(KPtr P, const int64_t* __restrict__ off, Layout lay, int64_t nw, const TE* __restrict__ E,
@@ -1929,6 +1944,10 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
     const dim3 gsp((unsigned)ceil_div(N * kG, kRows), (unsigned)ceil_div(R, std::min(b, 16)));
     switch (b) {
       case 1:
+        if (!use_spmv_one<TV, TE>(ctx)) {
+          k_spmv<TV, TE, 1, RS><<<gsp, kRows, 0, s>>>(P, ri, ctx->offd.colmap, E, src, dst, Bv);
+          break;
+        }
         k_spmv_one<TV, TE, RS><<<(unsigned)ceil_div(ctx->nw * kG, kOneThreads), kOneThreads, 0, s>>>(
             P, ctx->off, ctx->offd, ctx->nw, E, src, dst, Bv);
         break;
