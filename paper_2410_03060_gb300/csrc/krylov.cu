@@ -374,9 +374,9 @@ __global__ void __launch_bounds__(256) k_spmv_t(KPtr P, const RowInfo* __restric
 // The column map is loaded one group of four ahead of its gathers.  The entries of E are the same
 // address for every thread of a wire (one transaction per warp).  Rows are taken eight at a time
 // (a wire has at most SWM_MAX_SEG - 1 rows).
-// With `order` (float64) the wires go in that order, sorted by (rows, columns) within windows: float64
-// multiply-adds set the time there, and a warp issues them for the largest row and column counts of its
-// wires.  Seven right-hand sides at 50,000 wires 0.97 -> 0.67 ms.
+// With `order` (float64, see row_order) the wires go in that order, sorted by (rows, columns) within windows:
+// float64 multiply-adds set the time there, and a warp issues them for the largest row and column counts of
+// its wires.  Seven right-hand sides at 50,000 wires 0.97 -> 0.67 ms.
 // MODE kStepW: a GMRES step (active right-hand sides only); kResW: the residual at the start of a
 // cycle, every right-hand side, source Y, result W = B - (y + E y); kPlainW: every right-hand side,
 // W = u + E u (the product on its own, for callers outside GMRES).
@@ -1131,6 +1131,25 @@ inline WireTile wire_tile(int R, int64_t nw) {
   t.gx = (unsigned)ceil_div(nw, t.WB);
   t.gy = (unsigned)ceil_div(R, t.RG);
   return t;
+}
+
+// The order in which a float64 wire-tiled product takes the wires (nullptr: as they lie).  Sorting pays where wires
+// share warps and the CTAs are many or few: a CTA of long wires alone keeps its SM busy after the others, and a
+// wire that fills its warps gains nothing.  Products of a solve as they lie and sorted: 300 wires x 6 1.94 and
+// 1.67 ms, 16,000 x 6 5.85 and 4.32, x 16 8.64 and 7.56; but 8,000 x 9 3.50 and 3.85 (0.94 waves of CTAs), 2,000 x
+// 16 2.07 and 2.41, 2,000 x 32 2.67 and 3.50, 4,000 x 48 5.95 and 6.18 ms (at 15,000 x 60 25.2 and 23.4).  Below
+// 128 wires the sort, 40 us a pattern, costs more than it saves.
+int row_order(swm_ctx* ctx, const WireTile& wt, const int32_t** order) {
+  *order = nullptr;
+  const int64_t ctas = (int64_t)wt.gx * wt.gy, wave = 2 * (int64_t)std::max(ctx->nsm, 1);
+  const bool pays = wt.RG <= 6    ? true
+                    : wt.RG <= 12 ? 10 * ctas <= 3 * wave || ctas >= wave
+                    : wt.RG < 32  ? 2 * ctas >= 3 * wave
+                                  : wt.RG % 32 != 0 && ctas >= 6 * wave;
+  if (ctx->nw < 128 || !pays) return SWM_OK;
+  SWM_TRY(ensure_row_order(ctx));
+  *order = ctx->worder;
+  return SWM_OK;
 }
 
 // Arrival of one right-hand side at the end of the dots pass of step j; the last one advances the
@@ -1935,6 +1954,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   constexpr int kWire = 64;  // k_spmv_w: wire-tiled, right-hand-side major, no transposed copy
   int rb = multi ? 8 : 1;
   const WireTile wt = wire_tile(R, ctx->nw);
+  const int32_t* order = nullptr;  // of the float64 wire-tiled products
 
   // res: the residual U = B - A Y of a cycle's start in the same form (every right-hand side)
   auto product = [&](cudaStream_t s, int b, auto res_tag) -> int {
@@ -1988,7 +2008,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
           }
         }
         k_spmv_w<TV, TE, RS ? kResW : kStepW, false><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-            P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+            P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, order);
         break;
       case kWire + 4:  // packed FP32x2 arithmetic, E expanded and the column map in shared memory
       case kWire + 5:  // the same with two CTAs per SM and a larger E budget
@@ -2016,7 +2036,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
           }
         }
         k_spmv_w<TV, TE, RS ? kResW : kStepW, false><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-            P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+            P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, order);
         break;
       case kWire + 1:  // the same with five CTAs per SM (fewer registers)
         if (ws->Xt) {
@@ -2024,10 +2044,10 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
                                                                                                         ws->Xt);
           SWM_LAUNCHED();
           k_spmv_w<TV, TE, RS ? kResW : kStepW, true, 5><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-              P, ctx->off, ctx->offd, ctx->nw, E, src, ws->Xt, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+              P, ctx->off, ctx->offd, ctx->nw, E, src, ws->Xt, dst, Bv, wt.RG, wt.WB, order);
         } else {
           k_spmv_w<TV, TE, RS ? kResW : kStepW, false, 5><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-              P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+              P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, order);
         }
         break;
       case kWire:
@@ -2037,10 +2057,10 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
                                                                                                         ws->Xt);
           SWM_LAUNCHED();
           k_spmv_w<TV, TE, RS ? kResW : kStepW, true><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-              P, ctx->off, ctx->offd, ctx->nw, E, src, ws->Xt, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+              P, ctx->off, ctx->offd, ctx->nw, E, src, ws->Xt, dst, Bv, wt.RG, wt.WB, order);
         } else {
           k_spmv_w<TV, TE, RS ? kResW : kStepW, false><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-              P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+              P, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, order);
         }
         break;
       default: k_spmv<TV, TE, 8, RS><<<gsp, kRows, 0, s>>>(P, ri, ctx->offd.colmap, E, src, dst, Bv); break;
@@ -2095,7 +2115,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
   };
   if (!persisted && multi) {
     if constexpr (std::is_same<TV, double>::value)
-      SWM_TRY(ensure_row_order(ctx));
+      SWM_TRY(row_order(ctx, wt, &order));
     else
       SWM_TRY(build_wire_order(ctx));  // form 75 (tuned or forced) takes the wires in this order
     const int64_t shape[6] = {N, R, (int64_t)sizeof(TV), (int64_t)sizeof(TE), P.chunk, restart};
@@ -2156,7 +2176,7 @@ int gmres_impl(swm_ctx* ctx, const TE* E, double tol, int restart, int max_iter,
     std::memset(&key, 0, sizeof(key));
     key.P = P;
     const void* ptrs[9] = {ctx->rowinfo, ctx->offd.colmap, E, U, Wv, V, ws->Xt, ctx->off,
-                           sizeof(TV) == 8 ? (const void*)ctx->worder : ctx->wrec};
+                           sizeof(TV) == 8 ? (const void*)order : ctx->wrec};
     for (int i = 0; i < 9; ++i) key.ptr[i] = ptrs[i];
     key.lay = ctx->offd;
     key.gx = g_chunk.x;
@@ -2563,9 +2583,7 @@ __global__ void __launch_bounds__(kRows) k_bi_check(BPtr B, const cplx<TV>* __re
 
 template <typename TV, typename TE>
 int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
-  if constexpr (std::is_same<TV, double>::value)
-    SWM_TRY(ensure_row_order(ctx));
-  else
+  if constexpr (std::is_same<TV, float>::value)
     SWM_TRY(build_wire_order(ctx));  // the order of product form 75, once per pattern
   cudaStream_t st = ctx->stream;
   const int R = ctx->n_rhs;
@@ -2642,6 +2660,8 @@ int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
   SWM_TRY(norms_of_b(ctx, ctx->Bv, sizeof(TV) == sizeof(double), B.bnorm));
   SWM_TRY(init_y(ctx, Y, sizeof(TV) == sizeof(double)));
   const WireTile wt = wire_tile(R, ctx->nw);
+  const int32_t* order = nullptr;
+  if constexpr (std::is_same<TV, double>::value) SWM_TRY(row_order(ctx, wt, &order));
   const int RQ = std::min(32, (int)ceil_div(R, 2));
   const int WBp = std::max(1, std::min(kWpMaxWires, 256 / RQ));
   const int T = std::max(8, std::min(64, (int)((48 * 1024 / sizeof(cplx<TV>)) / (xst + 1)) / 8 * 8));
@@ -2666,7 +2686,7 @@ int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
       }
     }
     k_spmv_w<TV, TE, RS ? kResW : kStepW, false><<<dim3(wt.gx, wt.gy), 256, 0, s>>>(
-        PP, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, sizeof(TV) == 8 ? ctx->worder : nullptr);
+        PP, ctx->off, ctx->offd, ctx->nw, E, src, nullptr, dst, Bv, wt.RG, wt.WB, order);
     SWM_LAUNCHED();
     return SWM_OK;
   };
@@ -2776,7 +2796,7 @@ int bicgstab_impl(swm_ctx* ctx, const TE* E, double tol, int max_iter) {
     std::memset(&gk, 0, sizeof(gk));
     gk.B = B;
     const void* ptrs[13] = {E, Y, Rv, Rh, Pv, Vv, Sv, Tv, ws->Xt, ctx->off, ws->kst, Bv,
-                            sizeof(TV) == 8 ? (const void*)ctx->worder : ctx->wrec};
+                            sizeof(TV) == 8 ? (const void*)order : ctx->wrec};
     for (int i = 0; i < 13; ++i) gk.ptr[i] = ptrs[i];
     gk.lay = ctx->offd;
     gk.bits = -(int64_t)(sizeof(TV) * 64 + sizeof(TE));
@@ -3592,38 +3612,40 @@ int bicgstab_solve(swm_ctx* ctx, double tol, int max_iter) {
 }
 
 int residual_f64_wire(swm_ctx* ctx, const c128* B, const c128* Y, c128* Rr, c128* Yt) {
-  SWM_TRY(ensure_row_order(ctx));
   KPtr P{};
   P.R = ctx->n_rhs;
   P.N = ctx->N;
   const WireTile wt = wire_tile(P.R, ctx->nw);
+  const int32_t* order = nullptr;
+  SWM_TRY(row_order(ctx, wt, &order));
   if (Yt) {
     // y right-hand-side minor first, so that the gathers of a wire's threads are contiguous
     k_rhs_minor<double, true><<<dim3((unsigned)ceil_div(P.N, 32), (unsigned)ceil_div(P.R, 32)), 256, 0,
                                 ctx->stream>>>(P, Y, Yt);
     SWM_LAUNCHED();
     k_spmv_w<double, c64, kResW, true><<<dim3(wt.gx, wt.gy), 256, 0, ctx->stream>>>(
-        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, Y, Yt, Rr, B, wt.RG, wt.WB, ctx->worder);
+        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, Y, Yt, Rr, B, wt.RG, wt.WB, order);
   } else {
     k_spmv_w<double, c64, kResW, false><<<dim3(wt.gx, wt.gy), 256, 0, ctx->stream>>>(
-        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, Y, nullptr, Rr, B, wt.RG, wt.WB, ctx->worder);
+        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, Y, nullptr, Rr, B, wt.RG, wt.WB, order);
   }
   SWM_LAUNCHED();
   return SWM_OK;
 }
 
 int product_f64(swm_ctx* ctx, int R, const c128* X, c128* Y) {
-  SWM_TRY(ensure_row_order(ctx));
   KPtr P{};
   P.R = R;
   P.N = ctx->N;
   const WireTile wt = wire_tile(R, ctx->nw);
+  const int32_t* order = nullptr;
+  SWM_TRY(row_order(ctx, wt, &order));
   if (ctx->prec == SWM_C128)
     k_spmv_w<double, c128, kPlainW, false><<<dim3(wt.gx, wt.gy), 256, 0, ctx->stream>>>(
-        P, ctx->off, ctx->offd, ctx->nw, (const c128*)ctx->Zp, X, nullptr, Y, nullptr, wt.RG, wt.WB, ctx->worder);
+        P, ctx->off, ctx->offd, ctx->nw, (const c128*)ctx->Zp, X, nullptr, Y, nullptr, wt.RG, wt.WB, order);
   else
     k_spmv_w<double, c64, kPlainW, false><<<dim3(wt.gx, wt.gy), 256, 0, ctx->stream>>>(
-        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, X, nullptr, Y, nullptr, wt.RG, wt.WB, ctx->worder);
+        P, ctx->off, ctx->offd, ctx->nw, (const c64*)ctx->Zp, X, nullptr, Y, nullptr, wt.RG, wt.WB, order);
   SWM_LAUNCHED();
   return SWM_OK;
 }
