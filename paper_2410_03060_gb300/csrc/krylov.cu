@@ -3181,7 +3181,19 @@ __global__ void __launch_bounds__(256) k_minor_to_major(int64_t N, int R, int xs
 // in form 74, 9.7 in 75, 8.7 in 76: the call took 2.48 ms with 74, 2.57 with 76 chosen by the product alone.
 constexpr int kTuneProducts = 32;
 constexpr double kOrderMs = 0.045;
-constexpr float kTuneAllMs = 0.1f;  // products up to which every form is timed
+
+// The forms worth timing (a first solve of a shape pays for each): over 146 systems of 30 to 120,000 wires, 4 to
+// 100 entries a row and 2 to 150 incidences, the best of them was on average within 0.9 % of the best of all nine
+// by that cost, at most 6 %.  Rows of twelve entries and more want form 76 or, on small clouds, 74; short rows 68 or
+// 74 up to a million multiply-adds a product, 68, 71 or 76 up to ten million, then 73 or 76.  All nine took the
+// first solve of 60,000 wires x 2 from 13.0 to 17.8 ms.
+std::vector<int> tuned_forms(int64_t nval, int64_t N, int R) {
+  if (nval >= 12 * N) return {76, 74};
+  const double work = (double)nval * R;
+  if (work < 1e6) return {68, 74};
+  if (work < 1e7) return {68, 71, 76};
+  return {73, 76};
+}
 
 int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
   cudaStream_t st = ctx->stream;
@@ -3300,19 +3312,20 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
     } else {
       bool packed = false;
       const bool had_pack = ctx->pack != nullptr;
-      SWM_TRY(build_wire_order(ctx));
-      SWM_TRY(ensure_pack(ctx, &packed));
-      // Each shape once untimed and once timed on b (the product is idempotent), the sorted forms first.
-      // Form 76 leads from 30,000 wires (by up to 4 on clusters), 74, 75 and 69 on smaller clouds; the others
-      // are timed while a product is short, where one of them can be the best and their timing costs little.
+      std::vector<int> forms = tuned_forms(ctx->offd.nval, N, R);
+      if (std::find(forms.begin(), forms.end(), 76) != forms.end()) {
+        SWM_TRY(ensure_pack(ctx, &packed));
+        if (!packed) {
+          forms = {68, 69, 70, 71, 72, 73, 74, 75};
+          SWM_TRY(build_wire_order(ctx));
+        }
+      }
+      // each form once untimed and once timed on b (the product is idempotent)
       cudaEvent_t e0, e1;
       SWM_CK(cudaEventCreate(&e0));
       SWM_CK(cudaEventCreate(&e1));
       double best = 0.0;
-      float shortest = 0.f;
-      for (int f : {76, 75, 73, 74, 69, 68, 70, 71, 72}) {
-        if (!packed && f == 76) continue;
-        if (packed && f != 73 && f < 75 && shortest > kTuneAllMs) break;
+      for (int f : forms) {
         form = f;
         SWM_TRY(product(st, Bt, Vv, std::true_type{}));
         SWM_CK(cudaEventRecord(e0, st));
@@ -3321,7 +3334,6 @@ int bicgstab_minor(swm_ctx* ctx, const c64* E, double tol, int max_iter) {
         SWM_CK(cudaEventSynchronize(e1));
         float ms = 0.f;
         SWM_CK(cudaEventElapsedTime(&ms, e0, e1));
-        if (shortest == 0.f || ms < shortest) shortest = ms;
         const double cost = kTuneProducts * ms + (f == 76 ? pack_ms(ctx) : f == 75 ? kOrderMs : 0.0);
         if (best == 0.0 || cost < best) {
           best = cost;
