@@ -2997,8 +2997,8 @@ __global__ void __launch_bounds__(256) k_bp_dir(BmPtr B, const c64* __restrict__
     return;
   }
   const bool f0 = a0 && B.fresh[c0], f1 = a1 && B.fresh[c1];
-  // a fresh half takes p = r (its rh is set to r) and an inactive half too: neither reads beta, omega, p
-  // or v, which hold nothing yet or what another solve left (zero times a NaN is a NaN)
+  // a fresh half takes p = r (its rh is set to r) and an inactive half too: with zeros in the place of beta,
+  // omega, p and v, which hold nothing yet or what another solve left (zero times a NaN is a NaN)
   const bool d0 = a0 && !f0, d1 = a1 && !f1;
   const c64 z = mkc(0.f, 0.f);
   const c64 be0 = d0 ? bp_sc(B, B.beta, c0) : z, be1 = d1 ? bp_sc(B, B.beta, c1) : z;
@@ -3007,8 +3007,8 @@ __global__ void __launch_bounds__(256) k_bp_dir(BmPtr B, const c64* __restrict__
   for (int64_t n = t.n0 + t.rl; n < t.n1; n += t.nrl) {
     const int64_t o = n * xst + c0;
     const float4 r = ld4(Rv + o), p = ld4(Pv + o), v = ld4(Vv + o);
-    st4(Out + o, f4(d0 ? lo(r) + be0 * (lo(p) - om0 * lo(v)) : lo(r),
-                    d1 ? hi(r) + be1 * (hi(p) - om1 * hi(v)) : hi(r)));
+    const c64 p0 = d0 ? lo(p) : z, p1 = d1 ? hi(p) : z, v0 = d0 ? lo(v) : z, v1 = d1 ? hi(v) : z;
+    st4(Out + o, f4(lo(r) + be0 * (p0 - om0 * v0), hi(r) + be1 * (p1 - om1 * v1)));
     if (f0 && f1) {
       st4(Rh + o, r);
     } else if (f0) {
