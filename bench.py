@@ -385,7 +385,7 @@ def roofline_of(cls, st, prof_ms, launches, prec, n_rhs, restart, steps, pk, per
         flops = st["fill_evals"] * FP32_FLOPS_PER_EVAL * steps
         peak = fp32_peak_tflops(pk) if prec != "c128" else 1.25
         ach = flops / (prof_ms * 1e-3) / 1e12
-        return {"kernel": "k_mutual_blocks_f32" if prec != "c128" else "k_mutual_blocks<double>", "bound": "alu",
+        return {"kernel": "k_mutual_blocks_f32" if prec != "c128" else "k_mutual_blocks_f64", "bound": "alu",
                 "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "per_launch_flops": flops / launches, "per_launch_ms": per_launch_ms,
                 "peak_source": ("FP32 peak = 152 SMs x 128 lanes x 2 flops x max SM clock" if prec != "c128"
@@ -397,7 +397,7 @@ def roofline_of(cls, st, prof_ms, launches, prec, n_rhs, restart, steps, pk, per
     work = b * steps
     ach = work / (prof_ms * 1e-3) / 1e9
     peak = pk.get("hbm_gbs", 6800.0)
-    names = {"apply": "block-sparse product, form %s (k_spmv_wa / k_spmv_wg / k_spmv_wm / k_spmv_wp / k_spmv_w / "
+    names = {"apply": "block-sparse product, form %s (k_spmv_pack / k_spmv_wa / k_spmv_wg / k_spmv_wm / k_spmv_wp / k_spmv_w / "
                       "k_spmv_t / k_spmv, timed per shape)" % st.get("step_rhs_block"),
              "transpose": "k_rhs_minor_all: pending vectors to incidence-minor order",
              "dots": "k_dots: delayed Gram-Schmidt inner products",

@@ -534,7 +534,7 @@ int swm_build(swm_ctx* ctx, double k, double r_c, int precision) {
   ctx->bf16 = precision == SWM_BF16;
   ctx->E16 = nullptr;
   ctx->pack = nullptr;
-  if (!ctx->side) {  // the build's second stream (pattern column maps, self blocks, far-field data)
+  if (!ctx->side) {  // the build's second stream (self blocks, their inverses, far-field data)
     SWM_CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
     SWM_CK(cudaEventCreateWithFlags(&ctx->side_ev[0], cudaEventDisableTiming));
     SWM_CK(cudaEventCreateWithFlags(&ctx->side_ev[1], cudaEventDisableTiming));

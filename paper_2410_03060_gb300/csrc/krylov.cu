@@ -38,7 +38,7 @@ constexpr int kRows = 256;  // CTA width of the vector kernels
 constexpr int kMinorR = 12;  // right-hand sides from which the large-system product reads them
                              // right-hand-side minor (one lane each)
 constexpr int kG = 8;       // lanes per scalar row in the block-sparse product
-constexpr int kMaxChunk = 2048;  // rows per CTA of the Gram-Schmidt kernels, at most
+constexpr int kMaxChunk = 2048;  // rows per CTA of the GMRES update, the staged dots and BiCGSTAB's passes, at most
 
 // A solve's workspace stays in the context only when all of its buffers exist: an allocation that fails
 // (or any other way out before `complete`) gives back what was there and forgets the workspace, so the

@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(128) k_invert_self(int64_t nw, const int32_t* 
 // rows q (up to 32), a lane a column of one of them: Z is symmetric bit for bit (Z_pq = Z_qp^T, stored twice by the
 // fill), so row i of Z_pq is column i of Z_qp, and the lanes of a warp read Z along the rows of q
 // (consecutive blocks are consecutive columns) and share the entries of Minv_q, each entry read once for
-// the whole row of E_pq.  Bound by HBM in float32.  A warp per block with a lane per entry read every
+// the whole row of E_pq.  Bound by its writes: the rows of E_pq are a wire's few entries (40 bytes), parts of
+// memory's lines, and the bytes it cannot do without pass at 0.26 of HBM.  A warp per block with a lane per entry read every
 // entry of Z and Minv_q m_q times and divided for its indices: 1,000,000 wires 4.14 -> 1.81 ms, entire
 // coupling of 1,000 wires 0.49 -> 0.25 ms.
 constexpr int kFormThreads = 128;

@@ -103,7 +103,7 @@ __device__ __forceinline__ void obs_frame(const double* obs, int stride, int o, 
 }
 
 // sinc(z) and cos(z), sin(z) = z sinc(z): Taylor series to z^12 for z^2 <= kSmallZ2 (first neglected
-// terms below 1e-19; segments of up to 0.086 wavelengths seen along their axis), else from the table.
+// terms below 1.3e-19; segments of up to 0.086 wavelengths seen along their axis), else from the table.
 constexpr double kSmallZ2 = 0.073;
 __device__ __forceinline__ void sinc_cos(double z, double* sinc, double* c) {
   const double x = z * z;
@@ -128,8 +128,9 @@ __device__ __forceinline__ void sinc_cos(double z, double* sinc, double* c) {
 // rooftops e^{2jz} and sinc(z), z = k r.t D / 2, from one pair of short series; the rooftops are
 // summed in Horner form, 4 instructions each.  About 45 + 26 per incidence against 180 per incidence
 // and wire with CUDA's sincos and a running phase factor: 10,000 wires, 2 incidences, 361 angles
-// 2.09 -> 0.71 ms; error against quadruple precision 1.46e-14 (3,000
-// wires at 12 angles) against 1.49e-14.
+// 2.09 -> 0.71 ms.  Error against 112-bit arithmetic, 1,500 wires at 240 angles, 8.2e-15 (with CUDA's sincos
+// 8.5e-15), 200 wires at 400 angles 3.75e-15 (3.72e-15); against a plain float64 evaluation 1.09e-14
+// (9.6e-15): that evaluation rounds k r.c by itself, as the former kernel did and this one does not.
 constexpr int kFFStage = 32;  // wires staged at a time
 template <int RB>
 __global__ void __launch_bounds__(kFFThreads) k_far_partial(Geo geo, int64_t nw, int64_t N, double k, int n_rhs,
