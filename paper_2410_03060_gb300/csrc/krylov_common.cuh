@@ -48,6 +48,7 @@ struct KPtr {
   int R, restart, nchunk, chunk;  // rows per CTA of the dots and cycle-start kernels
   int nuchunk, uchunk;             // rows per CTA of the update
   int max_iter;
+  int pad;  // no holes: captured steps are kept by the bytes of this struct
   int64_t N;
   double tol;
   float qs, qsi;  // scale of a basis stored in half precision (sqrt(N)) and its inverse, else 1
